@@ -45,12 +45,18 @@ template <typename T> __device__ __forceinline__ T cmk(decltype(T::x) a, decltyp
 }
 template <typename T> __device__ __forceinline__ T cadd(T a, T b) { return cmk<T>(a.x + b.x, a.y + b.y); }
 template <typename T> __device__ __forceinline__ T csub(T a, T b) { return cmk<T>(a.x - b.x, a.y - b.y); }
+// Rounded products and fused multiply-adds, written out so that every kernel that holds a
+// transform rounds it alike (the compiler is free to choose which product of a sum it fuses).
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
 template <typename T> __device__ __forceinline__ T cmul(T a, T b) {
-  return cmk<T>(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+  return cmk<T>(fma_rn(a.x, b.x, -mul_rn(a.y, b.y)), fma_rn(a.x, b.y, mul_rn(a.y, b.x)));
 }
 // a * conj(b)
 template <typename T> __device__ __forceinline__ T cmulc(T a, T b) {
-  return cmk<T>(a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y);
+  return cmk<T>(fma_rn(a.x, b.x, mul_rn(a.y, b.y)), fma_rn(a.y, b.x, -mul_rn(a.x, b.y)));
 }
 template <typename T> __device__ __forceinline__ T cconj(T a) { return cmk<T>(a.x, -a.y); }
 template <typename T> __device__ __forceinline__ T cscale(T a, decltype(T::x) s) { return cmk<T>(a.x * s, a.y * s); }

@@ -26,7 +26,7 @@
 // DCT-IV through a half-length FFT with pre- and post-twiddles).
 #pragma once
 
-#include "axis_pass.cuh"
+#include "pairs.cuh"
 
 namespace pc {
 namespace lean {
@@ -111,24 +111,6 @@ struct Geo {
   static constexpr int N = 2 * M;   // real line length
 };
 
-// e^{-2 pi i/3}: cos = -1/2, sin = -sqrt(3)/2
-__device__ __forceinline__ void dft3(float2 &a0, float2 &a1, float2 &a2) {
-  const float c = 0.86602540378443864676f;
-  const float2 s = make_float2(a1.x + a2.x, a1.y + a2.y);
-  const float2 d = make_float2(a1.x - a2.x, a1.y - a2.y);
-  const float2 t = make_float2(a0.x - 0.5f * s.x, a0.y - 0.5f * s.y);
-  a0 = make_float2(a0.x + s.x, a0.y + s.y);
-  // y1 = t - i c d, y2 = t + i c d
-  a1 = make_float2(t.x + c * d.y, t.y - c * d.x);
-  a2 = make_float2(t.x - c * d.y, t.y + c * d.x);
-}
-
-template <int R>
-__device__ __forceinline__ void dft_r(float2 *v) {
-  if constexpr (R == 3) dft3(v[0], v[1], v[2]);
-  else small_dft<float2, R, false>(v, nullptr, 0);
-}
-
 // Stage s of the forward FFT on every line of the tile: thread (line l, lane u) runs the
 // butterflies j = u + T b, b < E / R. Butterfly j reads slots j + r M/R, multiplies them by
 // w_{Ns R}^{r (j mod Ns)}, runs a radix-R DFT and writes slot (j / Ns) Ns R + (j mod Ns) + r Ns.
@@ -161,7 +143,7 @@ __device__ __forceinline__ void stage(float2 *buf, int u, int l, const float2 *_
 #pragma unroll
       for (int r = 1; r < R; ++r) v[b * R + r] = cmul(v[b * R + r], __ldg(tw + r * kk));
     }
-    dft_r<R>(v + b * R);
+    dft_small<R>(v + b * R);
   }
   __syncthreads();
   float2 *wr = buf + l;
@@ -193,151 +175,28 @@ __device__ __noinline__ void fft_all(float2 *buf, int u, int l, const float2 *__
   fft<M, V, 0>(buf, u, l, tw, pre);
 }
 
-// Natural coefficient index -> position in the pass's coefficient layout (DST-II reversed).
-template <int FAM>
-__device__ __forceinline__ int coef_pos(int kind, int n, int i) {
-  return (FAM == 1 && kind == KIND_DD) ? n - 1 - i : i;
-}
-
-// The four coefficient positions of pair k (k in [0, M/2)) in the order fwd_pair and inv_pair
-// use: family 0 the packed real DFT [X0, X_{n/2}, Re X1, Im X1, ...] (k = 0: X0, X_{n/2} and
-// the self-paired V_{M/2}); family 1 X_k, X_{n-k}, X_{M-k}, X_{M+k} (k = 0: X_0, X_M, X_{M/2},
-// X_{n-M/2}), DST-II reversed; family 2 X_2q, X_{n-1-2q} for q = k and q = M - 1 - k.
-template <int M, int FAM>
-__device__ __forceinline__ void pair_positions(int k, int kind, int (&pos)[4]) {
-  constexpr int n = 2 * M;
-  if constexpr (FAM == 2) {
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int q = h == 0 ? k : M - 1 - k;
-      pos[2 * h] = 2 * q;
-      pos[2 * h + 1] = n - 1 - 2 * q;
-    }
-  } else if constexpr (FAM == 0) {
-    if (k == 0) { pos[0] = 0; pos[1] = 1; pos[2] = M; pos[3] = M + 1; }
-    else { pos[0] = 2 * k; pos[1] = 2 * k + 1; pos[2] = 2 * (M - k); pos[3] = 2 * (M - k) + 1; }
-  } else {
-    const int i0 = (k == 0) ? 0 : k, i1 = (k == 0) ? M : n - k, i2 = (k == 0) ? M / 2 : M - k,
-              i3 = (k == 0) ? n - M / 2 : M + k;
-    pos[0] = coef_pos<FAM>(kind, n, i0);
-    pos[1] = coef_pos<FAM>(kind, n, i1);
-    pos[2] = coef_pos<FAM>(kind, n, i2);
-    pos[3] = coef_pos<FAM>(kind, n, i3);
-  }
-}
-
-// Forward post-processing of pair k (k in [0, M/2)) of line l: the four coefficients it
-// yields, as (position, value). Family 0: real DFT in packed order [X0, X_{n/2}, Re X1, Im X1,
-// ...]; family 1: DCT-II (DST-II reversed); family 2: DCT-IV / DST-IV of slots k and M - 1 - k.
+// Forward post-processing of pair k (k in [0, M/2)) of line l: its four coefficients (pairs.cuh).
 template <int M, int V, int FAM>
 __device__ __forceinline__ void fwd_pair(const float2 *buf, int l, int k, int kind, const float2 *__restrict__ tw,
                                          int (&pos)[4], float (&val)[4]) {
   constexpr int LP = Geo<M, V>::LP;
-  pair_positions<M, FAM>(k, kind, pos);
-  if constexpr (FAM == 2) {
-    const float2 *tp = tw + tw_dct4post(M);
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int q = h == 0 ? k : M - 1 - k;
-      const float2 y = cmul(buf[q * LP + l], __ldg(tp + q));
-      val[2 * h] = y.x;
-      val[2 * h + 1] = (kind == KIND_ND) ? -y.y : y.y;
-    }
-    return;
-  }
-  const float2 *wq = tw + tw_quarter(M);
-  float2 Vk, Vm;   // V_k and V_{M-k} of the real DFT of the (reordered) line
-  if (k == 0) {
-    const float2 z0 = buf[l], zh = buf[(M / 2) * LP + l];
-    const float V0 = z0.x + z0.y, VM = z0.x - z0.y;
-    Vm = make_float2(zh.x, -zh.y);   // V_{M/2} = conj Z_{M/2}
-    if constexpr (FAM == 0) {
-      val[0] = V0;
-      val[1] = VM;
-      val[2] = Vm.x;
-      val[3] = Vm.y;
-    } else {
-      const float2 th = cmul(Vm, __ldg(wq + M / 2));
-      val[0] = V0;
-      val[1] = __ldg(wq + M).x * VM;
-      val[2] = th.x;
-      val[3] = -th.y;
-    }
-    return;
-  }
-  const float2 zk = buf[k * LP + l], zm = buf[(M - k) * LP + l];
-  // V_k = E + w^k O, V_{M-k} = conj(E - w^k O); E = (Z_k + conj Z_{M-k})/2, O = -i (Z_k - conj Z_{M-k})/2
-  const float2 Eh = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));
-  const float2 O = make_float2(0.5f * (zk.y + zm.y), -0.5f * (zk.x - zm.x));
-  const float2 Ow = cmul(O, __ldg(tw + tw_rdft(M) + k));
-  Vk = make_float2(Eh.x + Ow.x, Eh.y + Ow.y);
-  Vm = make_float2(Eh.x - Ow.x, Ow.y - Eh.y);
-  if constexpr (FAM == 0) {
-    val[0] = Vk.x;
-    val[1] = Vk.y;
-    val[2] = Vm.x;
-    val[3] = Vm.y;
-  } else {
-    // t = e^{-i pi k/(2n)} V_k: X_k = Re t, X_{n-k} = -Im t
-    const float2 tk = cmul(Vk, __ldg(wq + k)), tm = cmul(Vm, __ldg(wq + M - k));
-    val[0] = tk.x;
-    val[1] = -tk.y;
-    val[2] = tm.x;
-    val[3] = -tm.y;
-  }
+  int qa, qb;
+  pair_positions<FAM>(M, k, kind, pos);
+  pair_slots<FAM>(M, k, qa, qb);
+  fwd_values<FAM>(buf[qa * LP + l], buf[qb * LP + l], M, k, kind, tw, val);
 }
 
-// Inverse pre-processing of pair k of line l from its four coefficients (the positions
-// fwd_pair gives, in the same order): writes the conjugated slots the forward FFT then
-// inverts (family 2: the slots themselves, DCT-IV being its own inverse up to 2/n).
+// Inverse pre-processing of pair k of line l from its four coefficients, into its two slots.
 template <int M, int V, int FAM>
 __device__ __forceinline__ void inv_pair(float2 *buf, int l, int k, int kind, const float2 *__restrict__ tw,
                                          const float (&val)[4]) {
   constexpr int LP = Geo<M, V>::LP;
-  if constexpr (FAM == 2) {
-    const float2 *t4 = tw + tw_dct4pre(M);
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int q = h == 0 ? k : M - 1 - k;
-      const float x0 = val[2 * h], x1 = val[2 * h + 1];   // X_2q, X_{n-1-2q}
-      const float2 z = (kind == KIND_ND) ? make_float2(x0, x1) : make_float2(x1, x0);
-      buf[q * LP + l] = cmul(z, __ldg(t4 + q));
-    }
-    return;
-  }
-  const float2 *wq = tw + tw_quarter(M);
-  if (k == 0) {
-    float a, b;
-    float2 xh;   // the self-paired coefficient V_{M/2}
-    if constexpr (FAM == 0) {
-      a = val[0];
-      b = val[1];
-      xh = make_float2(val[2], val[3]);
-    } else {
-      const float2 wM = __ldg(wq + M);
-      a = val[0];
-      b = val[1] * wM.x - val[1] * wM.y;                      // Re V_M, V_M = (X_M - i X_M) conj(wq_M)
-      xh = cmulc(make_float2(val[2], -val[3]), __ldg(wq + M / 2));
-    }
-    buf[l] = make_float2(0.5f * (a + b), -0.5f * (a - b));  // conj Z_0
-    buf[(M / 2) * LP + l] = xh;                               // conj Z_{M/2} = V_{M/2}
-    return;
-  }
-  float2 xk, xm;   // V_k, V_{M-k}
-  if constexpr (FAM == 0) {
-    xk = make_float2(val[0], val[1]);
-    xm = make_float2(val[2], val[3]);
-  } else {
-    // V_i = (X_i - i X_{n-i}) e^{+i pi i/(2n)}
-    xk = cmulc(make_float2(val[0], -val[1]), __ldg(wq + k));
-    xm = cmulc(make_float2(val[2], -val[3]), __ldg(wq + M - k));
-  }
-  // Z_k = E + i O, Z_{M-k} = conj(E - i O); E = (V_k + conj V_{M-k})/2, O = (V_k - conj V_{M-k}) conj(w^k)/2
-  const float2 Eh = make_float2(0.5f * (xk.x + xm.x), 0.5f * (xk.y - xm.y));
-  const float2 D = make_float2(0.5f * (xk.x - xm.x), 0.5f * (xk.y + xm.y));
-  const float2 O = cmulc(D, __ldg(tw + tw_rdft(M) + k));
-  buf[k * LP + l] = make_float2(Eh.x - O.y, -(Eh.y + O.x));        // conj(E + i O)
-  buf[(M - k) * LP + l] = make_float2(Eh.x + O.y, Eh.y - O.x);     // E - i O
+  int qa, qb;
+  float2 za, zb;
+  pair_slots<FAM>(M, k, qa, qb);
+  inv_values<FAM>(val, M, k, kind, tw, za, zb);
+  buf[qa * LP + l] = za;
+  buf[qb * LP + l] = zb;
 }
 
 // ----------------------------------------------------------------------------- global I/O
@@ -613,7 +472,7 @@ __device__ __noinline__ void body_layout(const PassArgs<float> &A, int tile, flo
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         int pos[4];
-        pair_positions<M, FAM>(pu + T * (i + h), kind, pos);
+        pair_positions<FAM>(M, pu + T * (i + h), kind, pos);
         load_pair<FAM, COL>(A, lr, pos, val[h]);
       }
 #pragma unroll

@@ -18,7 +18,7 @@
 #include <cstring>
 #include <vector>
 
-#include "numeric.cuh"
+#include "dfloat.cuh"
 #include "pc_internal.cuh"
 
 namespace pc {
@@ -306,33 +306,6 @@ __device__ __forceinline__ VBlock tile_block(const GridDev &g, unsigned b) {
   return VBlock{b, 0u, 0u, (unsigned)g.nblk, 1u, 1u};
 }
 
-// ----------------------------------------------------------------------------- double-float
-// Unevaluated FP32 pairs (hi + lo, struct DF above) with error-free transformations (Knuth's TwoSum, Dekker's
-// product through fma); the _rn intrinsics keep the compiler from contracting them.
-__device__ __forceinline__ DF df_of(double v) {
-  DF r;
-  split_f64(v, r.hi, r.lo);
-  return r;
-}
-__device__ __forceinline__ DF df_neg(DF a) { return DF{-a.hi, -a.lo}; }
-__device__ __forceinline__ DF df_add(DF a, DF b) {
-  const float s = __fadd_rn(a.hi, b.hi);
-  const float z = __fsub_rn(s, a.hi);
-  float e = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, z)), __fsub_rn(b.hi, z));
-  e = __fadd_rn(e, __fadd_rn(a.lo, b.lo));
-  const float h = __fadd_rn(s, e);
-  return DF{h, __fsub_rn(e, __fsub_rn(h, s))};
-}
-__device__ __forceinline__ DF df_sub(DF a, DF b) { return df_add(a, df_neg(b)); }
-__device__ __forceinline__ DF df_mul(DF a, DF b) {
-  const float p = __fmul_rn(a.hi, b.hi);
-  float e = __fmaf_rn(a.hi, b.hi, -p);
-  e = __fmaf_rn(a.hi, b.lo, e);
-  e = __fmaf_rn(a.lo, b.hi, e);
-  const float h = __fadd_rn(p, e);
-  return DF{h, __fsub_rn(e, __fsub_rn(h, p))};
-}
-
 // ----------------------------------------------------------------------------- divergence
 // s = D_h U / (beta dt) (FP64; as an FP32 pair in double-float arithmetic on the mixed path),
 // its FP32 copy; want_sums 1: sum(s) and the mean, 2: also sum(s^2) (statistics).
@@ -525,17 +498,12 @@ __device__ __forceinline__ void neighbours(const GridDev &g, const double *p, co
   else pr = g.hi_kind[a] ? -pc : pc;
 }
 
-// A stored value as a double-float pair: FP64 values are split exactly as split_f64 does,
-// pairs are taken as they are.
-__device__ __forceinline__ DF to_df(double v) { return df_of(v); }
-__device__ __forceinline__ DF to_df(float2 v) { return DF{v.x, v.y}; }
-__device__ __forceinline__ DF df_neg_(DF a) { return DF{-a.hi, -a.lo}; }
 // Ghost value beyond a non-periodic end (GridDev lo_kind / hi_kind): from the edge value dc, or
 // the value at inner (the next point inward, which the end mirrors on a vertex grid).
 template <typename PV>
 __device__ __forceinline__ DF ghost_df(int kind, DF dc, const PV *__restrict__ p, int inner) {
   if (kind == 0) return dc;
-  if (kind == 1) return df_neg_(dc);
+  if (kind == 1) return df_neg(dc);
   if (kind == 2) return to_df(p[inner]);
   return DF{0.0f, 0.0f};
 }
@@ -616,13 +584,13 @@ __device__ __forceinline__ void residual_body(unsigned b, const GridDev &g, cons
         // the differences first: pl - dc and pr - dc cancel before any rounding of the sum
         // (forming pl + pr first raised the refinement floor: p 9.4e-13 from the FP64 path on
         // the channel instead of 1.5e-14)
-        const DF t = df_add(df_sub(pl, dc), df_sub(pr, dc));
-        acc = df_add(acc, df_mul(t, DF{g.ih2_hi[a], g.ih2_lo[a]}));
+        const DF t = second_difference(pl, dc, pr, DF{g.ih2_hi[a], g.ih2_lo[a]});
+        acc = a == 0 ? t : df_sum(acc, t);
       }
       DF sc = to_df(s[c]);
       if (rs.rule && rs.k == 0) smx = fmaxf(smx, fabsf(sc.hi));
-      if (SINGULAR) sc = df_sub(sc, mean);
-      const DF v = df_sub(sc, acc);
+      if (SINGULAR) sc = df_diff(sc, mean);
+      const DF v = residual_of(sc, acc);
       if (WRITE_R) r[c] = v.hi;
       if (rs.rule) rmx = fmaxf(rmx, fabsf(v.hi));
       if (NORM) {
@@ -649,7 +617,11 @@ __global__ void residual_kernel(GridDev g, const SV *__restrict__ s, const PV *_
                                 float *__restrict__ r, DevStats *stats, double *res2,
                                 double *partials, unsigned int *counter, RefineStep rs) {
   pdl_enter();
-  if (rs.rule == 1 && refine_stopped_before(stats, rs.k, rs.tol)) return;   // the refinement already ended
+  // the refinement already ended: one reader per CTA where many CTAs would queue for the norms'
+  // cache line, else every thread (no barrier: 0.4 us less on the few CTAs of a 128^2 grid)
+  if (rs.rule == 1 && rs.k > 0 &&
+      (gridDim.x >= 512 ? cta_refine_stopped_before(stats, rs.k, rs.tol) : refine_stopped_before(stats, rs.k, rs.tol)))
+    return;
   const int c = rs.chunk > 1 ? rs.chunk : 1;
   const int b0 = blockIdx.x * c, b1 = min(b0 + c, g.nblk);
   float rmx = 0.0f, smx = 0.0f;
@@ -1154,7 +1126,7 @@ __global__ void batch_residual(const BatchProblem *__restrict__ P, const int *__
   const BatchProblem &q = P[pi];
   const float2 *s2 = reinterpret_cast<const float2 *>(q.s64);
   const bool rule = q.tol > 0.0f;
-  if (rule && refine_stopped_before(q.ds, k, q.tol)) return;
+  if (rule && k > 0 && cta_refine_stopped_before(q.ds, k, q.tol)) return;
   const RefineStep rs{k, rule ? 2 : 0, q.tol, 1};
   const int b0 = (int)(blockIdx.x - seg[pi]) * kResidualChunk;
   const int b1 = min(b0 + kResidualChunk, q.g.nblk);
