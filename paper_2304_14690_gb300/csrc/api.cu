@@ -210,7 +210,8 @@ static pc_status alloc_workspace(Plan *p, cudaStream_t st) {
   } else {
     if (plan_alloc(p, (void **)&p->ut64, dd * N * 8) != PC_OK) return PC_ERR_OUT_OF_MEMORY;
   }
-  if (cudaMemsetAsync(p->counters, 0, 16 * sizeof(unsigned int), st) != cudaSuccess)
+  if (cudaMemsetAsync(p->counters, 0, 16 * sizeof(unsigned int), st) != cudaSuccess ||
+      cudaMemsetAsync(p->dstats, 0, sizeof(DevStats), st) != cudaSuccess)
     return fail(PC_ERR_CUDA, "counter reset failed");
   if (cudaStreamCreateWithFlags(&p->cap_stream, cudaStreamNonBlocking) != cudaSuccess)
     return fail(PC_ERR_CUDA, "stream creation failed");

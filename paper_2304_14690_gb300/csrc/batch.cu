@@ -33,14 +33,14 @@ struct PassLaunch {
   int nitems = 0;
   int emax = 1;          // largest slots per thread among the items' passes (kernel instance)
   size_t smem = 0;       // the pass body's shared memory (the largest item's)
-  int lean = 0;          // 0: general passes; else the lean kernel id (lean_pass.cuh)
+  int lean = 0;          // 0: general passes; 1-6 the lean kernel id (lean_pass.cuh); 7 looped passes
   int pass = 0;          // the pass of the solve: launches of one pass run side by side
 };
 
 // Auxiliary streams and events that run the launches of one batched pass side by side (they
 // transform disjoint problems), joined back into the caller's stream before the next pass. In a
 // captured graph they become parallel branches.
-constexpr int kForkWays = 6;
+constexpr int kForkWays = 7;
 struct Fork {
   cudaStream_t aux[kForkWays] = {};
   cudaEvent_t fork = nullptr, join[kForkWays] = {};
@@ -205,9 +205,9 @@ pc_status build_passes(Exec *e) {
     std::vector<PassLaunch> launches;
     for (size_t k = 0; k < npass; ++k) {
       struct Entry { long long key; int ai; long long tiles; };
-      // one launch per kernel: the general passes, and the lean passes of each lean kernel
-      std::vector<Entry> list[7];
-      PassLaunch pl[7];
+      // one launch per kernel: the general passes, the lean passes of each lean kernel, the looped ones
+      std::vector<Entry> list[8];
+      PassLaunch pl[8];
       for (const auto &ps : specs) {
         if (k >= ps.second.size()) continue;
         PassArgs<float> A;
@@ -217,7 +217,7 @@ pc_status build_passes(Exec *e) {
         PC_TRY(build_pass<float>(ps.first, ps.second[k], A, tiles, threads, smem, kBatchThreads));
         const bool pow2 = (A.M & (A.M - 1)) == 0;
         const long long key = ((long long)pass_family(A.kind) * 2 + (pow2 ? 0 : 1)) * 65536 + (65535 - A.M);
-        const int c = A.lean;
+        const int c = A.loop ? 7 : A.lean;
         list[c].push_back(Entry{key, (int)args.size(), tiles});
         args.push_back(A);
         pl[c].smem = std::max(pl[c].smem, smem);
@@ -225,7 +225,7 @@ pc_status build_passes(Exec *e) {
         pl[c].lean = c;
         pl[c].pass = (int)k;
       }
-      for (int c = 0; c < 7; ++c) {
+      for (int c = 0; c < 8; ++c) {
         if (list[c].empty()) continue;
         std::stable_sort(list[c].begin(), list[c].end(), [](const Entry &a, const Entry &b) { return a.key < b.key; });
         pl[c].items_off = (int)items.size();
@@ -300,9 +300,11 @@ pc_status record_exec(Exec *e, cudaStream_t st, Plan *prof = nullptr) {
           ls = e->fork->aux[i - a - 1];
           PC_CUDA_TRY(cudaStreamWaitEvent(ls, e->fork->fork, 0));
         }
-        if (pl.lean) {
-          PassArgs<float> none;
-          memset(&none, 0, sizeof(none));
+        PassArgs<float> none;
+        memset(&none, 0, sizeof(none));
+        if (pl.lean == 7) {
+          PC_TRY(launch_loop(none, e->dargs, e->ditems + pl.items_off, (unsigned)pl.nitems, pl.smem, ls));
+        } else if (pl.lean) {
           PC_TRY(launch_lean(pl.lean, none, e->dargs, e->ditems + pl.items_off, (unsigned)pl.nitems, kBatchThreads, pl.smem, ls));
         } else {
           PC_TRY(launch_batched_f32(e->dargs, e->ditems + pl.items_off, pl.nitems, kBatchThreads, pl.smem, pl.emax, ls));

@@ -65,6 +65,58 @@ __device__ __forceinline__ DF residual_of(DF s, DF acc) {
   return DF{h, __fsub_rn(v.lo, __fsub_rn(h, v.hi))};
 }
 
+// Two independent values per operation: the packed FP32 instructions of sm_103a, each half rounded
+// as the scalar operation rounds it.
+struct F2 { unsigned long long v; };
+__device__ __forceinline__ F2 f2_pack(float a, float b) {
+  F2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void f2_unpack(F2 a, float &x, float &y) { asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(a.v)); }
+__device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
+  F2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
+  F2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F2 f2_fma(F2 a, F2 b, F2 c) {
+  F2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+  return r;
+}
+// a - b as fma(b, -1, a): one rounding, the same as the subtraction's.
+__device__ __forceinline__ F2 f2_sub(F2 a, F2 b) { return f2_fma(b, f2_pack(-1.0f, -1.0f), a); }
+struct DF2 { F2 hi, lo; };
+__device__ __forceinline__ DF2 df2_of(DF a, DF b) { return DF2{f2_pack(a.hi, b.hi), f2_pack(a.lo, b.lo)}; }
+// df_sum, df_sub and second_difference on two points at a time, operation by operation.
+__device__ __forceinline__ DF2 df2_sum(DF2 a, DF2 b) {
+  const F2 s = f2_add(a.hi, b.hi), z = f2_sub(s, a.hi);
+  const F2 e = f2_add(f2_sub(a.hi, f2_sub(s, z)), f2_sub(b.hi, z));
+  return DF2{s, f2_add(e, f2_add(a.lo, b.lo))};
+}
+__device__ __forceinline__ DF2 df2_diff(DF2 a, DF2 b) {   // with -b in place of b: a + (-b) = a - b
+  const F2 s = f2_sub(a.hi, b.hi), z = f2_sub(s, a.hi);
+  const F2 e = f2_sub(f2_sub(a.hi, f2_sub(s, z)), f2_add(b.hi, z));
+  return DF2{s, f2_add(e, f2_sub(a.lo, b.lo))};
+}
+__device__ __forceinline__ DF2 df2_norm(DF2 v) {
+  const F2 h = f2_add(v.hi, v.lo);
+  return DF2{h, f2_sub(v.lo, f2_sub(h, v.hi))};
+}
+__device__ __forceinline__ DF2 second_difference2(DF2 pl, DF2 pc, DF2 pr, DF ih2) {
+  const DF2 t = df2_sum(df2_norm(df2_diff(pl, pc)), df2_norm(df2_diff(pr, pc)));
+  const F2 hh = f2_pack(ih2.hi, ih2.hi), hl = f2_pack(ih2.lo, ih2.lo);
+  const F2 p = f2_mul(t.hi, hh);
+  F2 e = f2_fma(t.hi, hh, f2_mul(p, f2_pack(-1.0f, -1.0f)));
+  e = f2_fma(t.hi, hl, e);
+  return DF2{p, f2_fma(t.lo, hh, e)};
+}
+
 // A stored value as a double-float pair: FP64 values are split exactly as split_f64 does, pairs
 // are taken as they are.
 __device__ __forceinline__ DF to_df(double v) { return df_of(v); }

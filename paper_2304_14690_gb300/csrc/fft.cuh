@@ -76,13 +76,6 @@ struct TileGeom {
   int tpl;   // threads per line (position stride)
 };
 
-// One FFT stage: radix R, current span Ns, twiddle stride M/(Ns R). j / Ns is a shift when Ns
-// is a power of two, else a multiply-high by magic = ceil(2^32/Ns) (exact for j < 2^16).
-struct StageInfo {
-  int R, Ns, stride_m, shift;   // shift < 0: use magic
-  unsigned magic;
-};
-
 // Table offsets inside one axis twiddle buffer (see AxisInfo).
 __host__ __device__ inline int tw_rdft(int M) { return M; }            // e^{-2 pi i k/n}, k=0..M
 __host__ __device__ inline int tw_quarter(int M) { return 2 * M + 1; }  // e^{-i pi k/(2n)}, k=0..M
@@ -133,6 +126,14 @@ __device__ __forceinline__ T w16(int e) {
   return cmk<T>(re, INV ? -im : im);
 }
 
+// a times w16(e) inside a radix-16 butterfly, with the product that each component fuses fixed: the
+// unrefined FP32 results have always had these bits.
+template <typename T, bool INV>
+__device__ __forceinline__ T cmul_w16(T a, T w, bool e6) {
+  const T p = cmul(a, w);
+  return cmk<T>(p.x, e6 ? p.y : fma_rn(a.y, w.x, mul_rn(a.x, w.y)));
+}
+
 // Small DFT of radix R on v[0..R-1], outputs in natural order. Radix 3 and 5 take their roots of
 // unity from the length-M FFT table (M divisible by R).
 template <typename T, int R, bool INV>
@@ -177,7 +178,7 @@ __device__ __forceinline__ void small_dft(T *v, const T *tw, int M) {
 #pragma unroll
       for (int j2 = 1; j2 < 4; ++j2) {
         if (j2 * k1 == 4) y[k1][j2] = rot4<T, INV>(y[k1][j2]);
-        else y[k1][j2] = cmul(y[k1][j2], w16<T, INV>(j2 * k1));
+        else y[k1][j2] = cmul_w16<T, INV>(y[k1][j2], w16<T, INV>(j2 * k1), j2 * k1 == 6);
       }
     }
 #pragma unroll

@@ -183,7 +183,7 @@ __device__ __forceinline__ void fwd_pair(const float2 *buf, int l, int k, int ki
   int qa, qb;
   pair_positions<FAM>(M, k, kind, pos);
   pair_slots<FAM>(M, k, qa, qb);
-  fwd_values<FAM>(buf[qa * LP + l], buf[qb * LP + l], M, k, kind, tw, val);
+  fwd_values<FAM>(buf[qa * LP + l], buf[qb * LP + l], M, k, kind, GlobalTables<float>{tw, nullptr, nullptr}, val);
 }
 
 // Inverse pre-processing of pair k of line l from its four coefficients, into its two slots.
@@ -194,7 +194,7 @@ __device__ __forceinline__ void inv_pair(float2 *buf, int l, int k, int kind, co
   int qa, qb;
   float2 za, zb;
   pair_slots<FAM>(M, k, qa, qb);
-  inv_values<FAM>(val, M, k, kind, tw, za, zb);
+  inv_values<FAM>(val, M, k, kind, GlobalTables<float>{tw, nullptr, nullptr}, za, zb);
   buf[qa * LP + l] = za;
   buf[qb * LP + l] = zb;
 }

@@ -9,6 +9,28 @@
 
 namespace pc {
 
+// A pass's tables: the wrappers' factors (tw, layout of fft.cuh's table offsets), the stage twiddles of
+// a looped pass and the eigenvalues of its axis, read from global memory through L1, or from a
+// CTA's shared memory (a barrier of the grid empties L1, so the resident kernel keeps them there).
+template <typename Real>
+struct GlobalTables {
+  using T = typename Cplx<Real>::T;
+  const T *w, *s;
+  const Real *l;
+  __device__ __forceinline__ T tw(int i) const { return __ldg(w + i); }
+  __device__ __forceinline__ T st(int i) const { return __ldg(s + i); }
+  __device__ __forceinline__ Real lam(int i) const { return __ldg(l + i); }
+};
+template <typename Real>
+struct SharedTables {
+  using T = typename Cplx<Real>::T;
+  const T *w, *s;
+  const Real *l;
+  __device__ __forceinline__ T tw(int i) const { return w[i]; }
+  __device__ __forceinline__ T st(int i) const { return s[i]; }
+  __device__ __forceinline__ Real lam(int i) const { return l[i]; }
+};
+
 // e^{-2 pi i/3}: cos = -1/2, sin = -sqrt(3)/2
 template <typename T>
 __device__ __forceinline__ void dft3(T &a0, T &a1, T &a2) {
@@ -94,19 +116,19 @@ __device__ __forceinline__ void pair_slots(int M, int k, int &qa, int &qb) {
 // Forward post-processing of pair k from its two slots za, zb of the FFT: the four coefficients at
 // pair_positions. Family 0: real DFT in packed order; family 1: DCT-II (DST-II reversed); family
 // 2: DCT-IV / DST-IV.
-template <int FAM, typename T>
-__device__ __forceinline__ void fwd_values(T za, T zb, int M, int k, int kind, const T *__restrict__ tw,
+template <int FAM, typename T, typename Tables>
+__device__ __forceinline__ void fwd_values(T za, T zb, int M, int k, int kind, const Tables &tb,
                                            decltype(T::x) (&val)[4]) {
   using R = decltype(T::x);
   if constexpr (FAM == 2) {
-    const T *tp = tw + tw_dct4post(M);
-    const T ya = cmul(za, __ldg(tp + k)), yb = cmul(zb, __ldg(tp + M - 1 - k));
+    const int tp = tw_dct4post(M);
+    const T ya = cmul(za, tb.tw(tp + k)), yb = cmul(zb, tb.tw(tp + M - 1 - k));
     val[0] = ya.x;
     val[1] = (kind == KIND_ND) ? -ya.y : ya.y;
     val[2] = yb.x;
     val[3] = (kind == KIND_ND) ? -yb.y : yb.y;
   } else {
-    const T *wq = tw + tw_quarter(M);
+    const int wq = tw_quarter(M);
     if (k == 0) {
       const R V0 = za.x + za.y, VM = za.x - za.y;
       const T Vh = cmk<T>(zb.x, -zb.y);   // V_{M/2} = conj Z_{M/2}
@@ -116,9 +138,9 @@ __device__ __forceinline__ void fwd_values(T za, T zb, int M, int k, int kind, c
         val[2] = Vh.x;
         val[3] = Vh.y;
       } else {
-        const T th = cmul(Vh, __ldg(wq + M / 2));
+        const T th = cmul(Vh, tb.tw(wq + M / 2));
         val[0] = V0;
-        val[1] = mul_rn(__ldg(wq + M).x, VM);
+        val[1] = mul_rn(tb.tw(wq + M).x, VM);
         val[2] = th.x;
         val[3] = -th.y;
       }
@@ -127,7 +149,7 @@ __device__ __forceinline__ void fwd_values(T za, T zb, int M, int k, int kind, c
     // V_k = E + w^k O, V_{M-k} = conj(E - w^k O); E = (Z_k + conj Z_{M-k})/2, O = -i (Z_k - conj Z_{M-k})/2
     const T Eh = cmk<T>((R)0.5 * (za.x + zb.x), (R)0.5 * (za.y - zb.y));
     const T O = cmk<T>((R)0.5 * (za.y + zb.y), (R)-0.5 * (za.x - zb.x));
-    const T Ow = cmul(O, __ldg(tw + tw_rdft(M) + k));
+    const T Ow = cmul(O, tb.tw(tw_rdft(M) + k));
     const T Vk = cmk<T>(Eh.x + Ow.x, Eh.y + Ow.y);
     const T Vm = cmk<T>(Eh.x - Ow.x, Ow.y - Eh.y);
     if constexpr (FAM == 0) {
@@ -137,7 +159,7 @@ __device__ __forceinline__ void fwd_values(T za, T zb, int M, int k, int kind, c
       val[3] = Vm.y;
     } else {
       // t = e^{-i pi k/(2n)} V_k: X_k = Re t, X_{n-k} = -Im t
-      const T tk = cmul(Vk, __ldg(wq + k)), tm = cmul(Vm, __ldg(wq + M - k));
+      const T tk = cmul(Vk, tb.tw(wq + k)), tm = cmul(Vm, tb.tw(wq + M - k));
       val[0] = tk.x;
       val[1] = -tk.y;
       val[2] = tm.x;
@@ -148,18 +170,18 @@ __device__ __forceinline__ void fwd_values(T za, T zb, int M, int k, int kind, c
 
 // Inverse pre-processing of pair k from its four coefficients: the conjugated slots the forward FFT
 // then inverts (family 2: the slots themselves, DCT-IV being its own inverse up to 2/n).
-template <int FAM, typename T>
+template <int FAM, typename T, typename Tables>
 __device__ __forceinline__ void inv_values(const decltype(T::x) (&val)[4], int M, int k, int kind,
-                                           const T *__restrict__ tw, T &za, T &zb) {
+                                           const Tables &tb, T &za, T &zb) {
   using R = decltype(T::x);
   if constexpr (FAM == 2) {
-    const T *t4 = tw + tw_dct4pre(M);
+    const int t4 = tw_dct4pre(M);
     const T a = (kind == KIND_ND) ? cmk<T>(val[0], val[1]) : cmk<T>(val[1], val[0]);   // X_2q, X_{n-1-2q}
     const T b = (kind == KIND_ND) ? cmk<T>(val[2], val[3]) : cmk<T>(val[3], val[2]);
-    za = cmul(a, __ldg(t4 + k));
-    zb = cmul(b, __ldg(t4 + M - 1 - k));
+    za = cmul(a, tb.tw(t4 + k));
+    zb = cmul(b, tb.tw(t4 + M - 1 - k));
   } else {
-    const T *wq = tw + tw_quarter(M);
+    const int wq = tw_quarter(M);
     if (k == 0) {
       R a, b;
       T xh;   // the self-paired coefficient V_{M/2}
@@ -168,10 +190,10 @@ __device__ __forceinline__ void inv_values(const decltype(T::x) (&val)[4], int M
         b = val[1];
         xh = cmk<T>(val[2], val[3]);
       } else {
-        const T wM = __ldg(wq + M);
+        const T wM = tb.tw(wq + M);
         a = val[0];
         b = fma_rn(val[1], wM.x, -mul_rn(val[1], wM.y));   // Re V_M, V_M = (X_M - i X_M) conj(wq_M)
-        xh = cmulc(cmk<T>(val[2], -val[3]), __ldg(wq + M / 2));
+        xh = cmulc(cmk<T>(val[2], -val[3]), tb.tw(wq + M / 2));
       }
       za = cmk<T>((R)0.5 * (a + b), (R)-0.5 * (a - b));   // conj Z_0
       zb = xh;                                            // conj Z_{M/2} = V_{M/2}
@@ -183,13 +205,13 @@ __device__ __forceinline__ void inv_values(const decltype(T::x) (&val)[4], int M
       xm = cmk<T>(val[2], val[3]);
     } else {
       // V_i = (X_i - i X_{n-i}) e^{+i pi i/(2n)}
-      xk = cmulc(cmk<T>(val[0], -val[1]), __ldg(wq + k));
-      xm = cmulc(cmk<T>(val[2], -val[3]), __ldg(wq + M - k));
+      xk = cmulc(cmk<T>(val[0], -val[1]), tb.tw(wq + k));
+      xm = cmulc(cmk<T>(val[2], -val[3]), tb.tw(wq + M - k));
     }
     // Z_k = E + i O, Z_{M-k} = conj(E - i O); E = (V_k + conj V_{M-k})/2, O = (V_k - conj V_{M-k}) conj(w^k)/2
     const T Eh = cmk<T>((R)0.5 * (xk.x + xm.x), (R)0.5 * (xk.y - xm.y));
     const T D = cmk<T>((R)0.5 * (xk.x - xm.x), (R)0.5 * (xk.y + xm.y));
-    const T O = cmulc(D, __ldg(tw + tw_rdft(M) + k));
+    const T O = cmulc(D, tb.tw(tw_rdft(M) + k));
     za = cmk<T>(Eh.x - O.y, -(Eh.y + O.x));   // conj(E + i O)
     zb = cmk<T>(Eh.x + O.y, Eh.y - O.x);      // E - i O
   }

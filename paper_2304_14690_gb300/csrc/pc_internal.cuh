@@ -16,14 +16,25 @@ namespace pc {
 enum AxisKind { KIND_PP = 0, KIND_NN = 1, KIND_DD = 2, KIND_ND = 3, KIND_DN = 4,
                 KIND_VNN = 5, KIND_VDD = 6, KIND_VND = 7, KIND_VDN = 8 };
 
-constexpr int kMaxRadices = 24;
+constexpr int kMaxRadices = 12;   // M <= 2048
 constexpr int kMaxK = 32;
 // Largest row count (cells, faces per axis, nodes) the kernels index with 32-bit row numbers.
 constexpr long long kMaxRows = (1LL << 31) - (1LL << 16);
 constexpr int kMaxRefine = 8;
 
 // Device-side status word values (written by kernels, read at the next sync point).
-enum DeviceFlag { FLAG_WLS_SINGULAR = 1, FLAG_KNN_SHORT = 2, FLAG_NONFINITE = 4 };
+enum DeviceFlag { FLAG_WLS_SINGULAR = 1, FLAG_KNN_SHORT = 2, FLAG_NONFINITE = 4, FLAG_TIMEOUT = 8 };
+
+// One FFT stage: radix R, current span Ns, twiddle stride M/(Ns R). j / Ns is a shift when Ns
+// is a power of two, else a multiply-high by magic = ceil(2^32/Ns) (exact for j < 2^16).
+struct StageInfo {
+  int R, Ns, stride_m, shift;   // shift < 0: use magic
+  unsigned magic;
+  // looped passes: butterflies per line M/R and their magic; stride_m is then the offset of the
+  // stage's twiddles
+  int mr;
+  unsigned mr_magic;
+};
 
 struct AxisInfo {
   int kind = 0;
@@ -45,6 +56,12 @@ struct AxisInfo {
   // twiddle of the real-to-real wrapper (kind dependent); [2M+1, 3M+1) DCT-IV pre twiddle.
   double2 *tw64 = nullptr;
   float2 *tw32 = nullptr;
+  // Schedule of the looped passes (loop_pass.cuh): 0 stages where the axis has none; the stages'
+  // twiddles follow the tables above in both precisions.
+  int loop_nst = 0;
+  StageInfo loop_st[kMaxRadices];
+  // FP64 passes: the looped ones until a slot count is set or the autotuner finds a faster one
+  bool loop64 = true;
   double *lam64 = nullptr;   // eigenvalue per spectral index (n entries)
   float *lam32 = nullptr;
 };
@@ -69,6 +86,7 @@ struct DevStats {
   // side by side, so that a kernel reads those of the first sweeps with one load
   alignas(16) float smax;
   float rmax[kMaxRefine + 1];
+  alignas(128) unsigned int bar[32];   // barrier of the cooperative solve (resident.cu): its own cache line
 };
 
 // The refinement's stopping rule on the stored max norms: residual k (after k sweeps) ends the
@@ -333,23 +351,6 @@ inline int grid_for(int64_t work, int threads) {
   return (int)b;
 }
 
-// Transform solves of a grid (poisson.cu): FP64 s -> p, and one FP32 solve whose source and
-// destination modes are those of passes.cuh (FP32 or FP64 source; FP64 set or accumulate).
-pc_status solve_fp64_grid(Plan *p, const double *s, double *pout, cudaStream_t st);
-// chunk: consecutive tiles per CTA (refinement sweeps that the stopping rule usually ends before
-// they start are launched with few CTAs, so a skipped sweep costs little)
-pc_status solve_fp32_grid(Plan *p, int src_mode, const void *s, int dst_mode, void *dst,
-                          cudaStream_t st, double *f64 = nullptr, RefineGate gate = RefineGate{nullptr, 0, 0.0f},
-                          int chunk = 1);
-// Drops the plan's captured CUDA graphs and batch executables (after a schedule change).
-void plan_drop_graphs(Plan *p);
-// ----------------------------------------------------------------------------- batches
-// Stages of the batched pipeline (one launch per stage for all problems of a batch).
-enum BatchStage {
-  BATCH_ZERO = 0, BATCH_PREP = 1, BATCH_TRANSFER = 2 /* +axis */, BATCH_DIVERGENCE = 5, BATCH_RESIDUAL = 6,
-  BATCH_GAUGE_SUM = 7, BATCH_FINALIZE = 8, BATCH_GRADIENT = 9, BATCH_STAGES = 10
-};
-
 // Cell-grid geometry and strides shared by the per-cell kernels (project.cu).
 struct GridDev {
   int dim;
@@ -368,6 +369,30 @@ struct GridDev {
   // 2^th_bits thread rows of cr rows each, gx tiles along the last axis, nblk blocks
   int rows, tw_bits, th_bits, cr, gx, nblk;
   const uint8_t *mask;          // RHS mask per cell (nonzero = flow domain), nullptr = none
+};
+
+// Transform solves of a grid (poisson.cu): FP64 s -> p, and one FP32 solve whose source and
+// destination modes are those of passes.cuh (FP32 or FP64 source; FP64 set or accumulate).
+pc_status solve_fp64_grid(Plan *p, const double *s, double *pout, cudaStream_t st);
+// chunk: consecutive tiles per CTA (refinement sweeps that the stopping rule usually ends before
+// they start are launched with few CTAs, so a skipped sweep costs little)
+pc_status solve_fp32_grid(Plan *p, int src_mode, const void *s, int dst_mode, void *dst,
+                          cudaStream_t st, double *f64 = nullptr, RefineGate gate = RefineGate{nullptr, 0, 0.0f},
+                          int chunk = 1);
+// Geometry of a plan's pressure grid for the cell kernels (project.cu).
+GridDev grid_dev(const Plan *p);
+// The refined FP32 solve as one cooperative kernel (resident.cu) where the plan and the arrays allow
+// it; taken says whether it was launched. s2 (nullable): the source as (hi, lo) pairs, else FP64 in
+// s64. The iterate is left in p->p2 and, in FP64, in pout.
+pc_status solve_resident(Plan *p, const double *s64, const float2 *s2, double *pout, int sweeps, bool adaptive,
+                         float tol, const GridDev &g, cudaStream_t st, bool &taken);
+// Drops the plan's captured CUDA graphs and batch executables (after a schedule change).
+void plan_drop_graphs(Plan *p);
+// ----------------------------------------------------------------------------- batches
+// Stages of the batched pipeline (one launch per stage for all problems of a batch).
+enum BatchStage {
+  BATCH_ZERO = 0, BATCH_PREP = 1, BATCH_TRANSFER = 2 /* +axis */, BATCH_DIVERGENCE = 5, BATCH_RESIDUAL = 6,
+  BATCH_GAUGE_SUM = 7, BATCH_FINALIZE = 8, BATCH_GRADIENT = 9, BATCH_STAGES = 10
 };
 
 // Per-problem parameters of a batched launch (device array, one entry per problem).

@@ -2,7 +2,8 @@
 //   1. forward 1D transforms along each axis in turn,
 //   2. division by the sum of the 1D eigenvalues of the central-difference Laplacian,
 //   3. backward 1D transforms.
-// One kernel launch per axis pass. The contiguous (last) axis is processed in row tiles, the
+// One kernel launch per axis pass; grids up to about a million cells take all the passes of an FP32
+// refined solve in one cooperative launch (resident.cu). The contiguous (last) axis is processed in row tiles, the
 // other axes in column tiles of W adjacent lines so that every global access is coalesced
 // without a transpose. The division is fused into the pass of axis 0, which does its forward
 // transform, the division and its inverse transform on the tile while it sits in shared memory.
@@ -17,6 +18,8 @@
 #include <vector>
 
 #include "lean_pass.cuh"
+#include "loop_pass.cuh"
+#include "resident.cuh"
 
 namespace pc {
 
@@ -62,6 +65,51 @@ bool vertex_axis_supported(int kind, int m) {
   return axis_length_supported(m);   // P-P and the quarter-wave pairs: length m, m even
 }
 
+// Schedule of the looped passes of a cell-grid axis: variant 0 of the length's compile-time pass
+// where it has one; else the power of two in radices of 16 and 8, then 3 and 5. Every stage has at
+// least two butterflies per line. Returns false where the axis has no looped pass.
+static bool loop_schedule(AxisInfo &ax) {
+  const int M = ax.M;
+  ax.loop_nst = 0;
+  if (pass_family(ax.kind) > 2 || (M & 1) || M < 6) return false;
+  int radix[kMaxRadices], nr = 0;
+  if (lean::length_ok(M)) {
+    for (int s = 0; lean::radix_of(M, 0, s) > 0; ++s) radix[nr++] = lean::radix_of(M, 0, s);
+  } else {
+    int m = M, two = 0;
+    while (m % 2 == 0) { m /= 2; ++two; }
+    if (m == 1 && two == 3) { radix[nr++] = 4; radix[nr++] = 2; two = 0; }   // M = 8
+    while (two >= 6 || two == 4) { radix[nr++] = 16; two -= 4; }
+    if (two == 5) { radix[nr++] = 8; two = 2; }
+    if (two) radix[nr++] = 1 << two;
+    while (m % 3 == 0) { radix[nr++] = 3; m /= 3; }
+    while (m % 5 == 0) { radix[nr++] = 5; m /= 5; }
+  }
+  int Ns = 1, off = 0;
+  for (int s = 0; s < nr; ++s) {
+    StageInfo &si = ax.loop_st[s];
+    si.R = radix[s];
+    si.Ns = Ns;
+    si.stride_m = off;
+    si.shift = ((Ns & (Ns - 1)) == 0) ? ilog2(Ns) : -1;
+    si.magic = (unsigned)(((1ULL << 32) + Ns - 1) / Ns);
+    si.mr = M / si.R;
+    if (si.mr < 2) return false;
+    si.mr_magic = (unsigned)(((1ULL << 32) + si.mr - 1) / si.mr);
+    if (Ns > 1) off += (si.R - 1) * Ns;
+    Ns *= si.R;
+  }
+  if (Ns != M) return false;
+  ax.loop_nst = nr;
+  return true;
+}
+static int loop_twiddles(const AxisInfo &ax) {
+  int n = 0;
+  for (int s = 0; s < ax.loop_nst; ++s)
+    if (ax.loop_st[s].Ns > 1) n += (ax.loop_st[s].R - 1) * ax.loop_st[s].Ns;
+  return n;
+}
+
 pc_status build_axis_tables(Plan *p) {
   for (int a = 0; a < p->dim; ++a) {
     AxisInfo &ax = p->ax[a];
@@ -76,6 +124,16 @@ pc_status build_axis_tables(Plan *p) {
     for (int k = 0; k <= M; ++k) put(tw_quarter(M), k, -pi * k / (2.0 * nt));
     for (int k = 0; k < M; ++k) put(tw_dct4pre(M), k, -pi * (4.0 * k + 1.0) / (4.0 * nt));
     for (int k = 0; k < M; ++k) put(tw_dct4post(M), k, -pi * k / (double)nt);
+    // stage twiddles of the looped passes, w_{Ns R}^{r k} = w_M^{r k M/(Ns R)} with k fast
+    loop_schedule(ax);
+    tw.resize(tw_total(M) + loop_twiddles(ax));
+    for (int s = 0; s < ax.loop_nst; ++s) {
+      const StageInfo &si = ax.loop_st[s];
+      if (si.Ns == 1) continue;
+      const int step = M / (si.Ns * si.R);
+      for (int r = 1; r < si.R; ++r)
+        for (int k = 0; k < si.Ns; ++k) tw[tw_total(M) + si.stride_m + (r - 1) * si.Ns + k] = tw[r * k * step];
+    }
     std::vector<float2> tw32(tw.size());
     for (size_t i = 0; i < tw.size(); ++i) tw32[i] = make_float2((float)tw[i].x, (float)tw[i].y);
     // eigenvalues per spectral index with the angle theta of each basis vector (th = theta/2):
@@ -115,33 +173,127 @@ pc_status build_axis_tables(Plan *p) {
   return PC_OK;
 }
 
+// The common part of a pass's arguments: axis, geometry, tables, source and destination.
 template <typename Real>
-pc_status build_pass(const Plan *p, const PassSpec &ps, PassArgs<Real> &A, long long &tiles, int &threads,
-                     size_t &smem, int batch_threads) {
+static void fill_pass(const Plan *p, const PassSpec &ps, PassArgs<Real> &A) {
   using T = typename Cplx<Real>::T;
-  const int axis = ps.axis;
-  const bool fwd = ps.fwd, div = ps.div, inv = ps.inv;
-  const int src_mode = ps.src_mode, dst_mode = ps.dst_mode;
-  const void *src = ps.src;
-  void *dst = ps.dst;
-  const AxisInfo &ax = p->ax[axis];
+  const AxisInfo &ax = p->ax[ps.axis];
   memset(&A, 0, sizeof(A));
-  A.axis = axis;
+  A.axis = ps.axis;
   A.kind = ax.kind;
   A.n = ax.n;
   A.M = ax.M;
+  A.tw = (const T *)(sizeof(Real) == 8 ? (const void *)ax.tw64 : (const void *)ax.tw32);
+  A.dim = p->dim;
+  int stride = 1;
+  for (int b = 0; b < p->dim; ++b) A.shape[b] = (int)p->n[b];
+  for (int b = ps.axis + 1; b < p->dim; ++b) stride *= (int)p->n[b];
+  A.stride = stride;
+  A.col = ps.axis != p->dim - 1;
+  A.do_fwd = ps.fwd;
+  A.do_div = ps.div;
+  A.do_inv = ps.inv;
+  for (int b = 0; b < p->dim; ++b)
+    A.lam[b] = (const Real *)(sizeof(Real) == 8 ? (const void *)p->ax[b].lam64 : (const void *)p->ax[b].lam32);
+  A.singular = p->singular;
+  A.src_mode = ps.src_mode;
+  A.src = ps.src;
+  A.dst_mode = ps.dst_mode;
+  A.dst = ps.dst;
+  A.out_scale = (Real)inv_scale(ax.M);
+  A.f64 = ps.f64;
+  A.gate = ps.gate;
+  A.chunk = ps.chunk > 1 ? ps.chunk : 1;
+}
+
+// Tiles of L lines of a pass.
+template <typename Real>
+static long long fill_tiles(const Plan *p, PassArgs<Real> &A, int L) {
+  long long tiles;
+  if (A.col) {
+    const long long outer = p->ncells / ((long long)A.stride * A.n);
+    A.inner = A.stride;
+    A.tiles_per_outer = (A.stride + L - 1) / L;
+    tiles = outer * A.tiles_per_outer;
+  } else {
+    const long long lines = p->ncells / A.n;
+    A.lines = (int)lines;
+    tiles = (lines + L - 1) / L;
+  }
+  A.L = L;
+  A.lbits = ilog2(L);
+  A.ntiles = (int)tiles;
+  return tiles;
+}
+
+// A looped pass with tiles of L lines (L a power of two).
+template <typename Real>
+static long long fill_loop(const Plan *p, const PassSpec &ps, PassArgs<Real> &A, int L) {
+  using T = typename Cplx<Real>::T;
+  const AxisInfo &ax = p->ax[ps.axis];
+  fill_pass<Real>(p, ps, A);
+  A.loop = 1;
+  A.fam = pass_family(ax.kind);
+  A.nst = ax.loop_nst;
+  for (int s = 0; s < ax.loop_nst; ++s) A.st[s] = ax.loop_st[s];
+  A.stw = A.tw + tw_total(ax.M);
+  A.half_magic = (unsigned)(((1ULL << 32) + ax.M / 2 - 1) / (ax.M / 2));
+  A.ls = loop::line_slots<Real>(ax.M, L);
+  return fill_tiles<Real>(p, A, L);
+}
+
+// Slots of a looped pass's tile: 2048 in FP32 (35 KB: six CTAs of 256 threads per SM) and 1024 in
+// FP64 in a launch of its own, up to 4096 on the resident CTAs.
+constexpr int kLoopSlots = 2048;
+
+static bool aligned16(const void *q) { return ((uintptr_t)q & 15) == 0; }
+
+// Whether the compile-time and the looped passes can run a pass: they move row tiles in 16-byte
+// accesses (16-byte aligned arrays), store forward coefficients as work and read inverse-only
+// coefficients in the pass precision.
+static bool quad_io(const Plan *p, const PassSpec &ps, bool fp32) {
+  const bool row = ps.axis == p->dim - 1;
+  return (!ps.fwd || ps.inv || ps.dst_mode == DST_WORK) && (!fp32 || ps.fwd || ps.src_mode != SRC_F64) &&
+         (!row || (aligned16(ps.src) && aligned16(ps.dst) && aligned16(ps.f64)));
+}
+
+template <typename Real>
+pc_status build_pass(const Plan *p, const PassSpec &ps, PassArgs<Real> &A, long long &tiles, int &threads,
+                     size_t &smem, int batch_threads) {
+  const int axis = ps.axis;
+  const AxisInfo &ax = p->ax[axis];
   const int M = ax.M;
   // slots per thread; 0 and 1 (FP32 only): variant 0 or 1 of the lean pass of the length
-  // (lean_pass.cuh) where it has one, else 4
-  int E = (sizeof(Real) == 8) ? ax.slots64 : ax.slots32;
-  // the lean passes move row tiles in 16-byte accesses (16-byte aligned arrays), store forward
-  // coefficients as FP32 work and read inverse-only coefficients in FP32
-  auto al16 = [](const void *q) { return ((uintptr_t)q & 15) == 0; };
-  const bool row = axis == p->dim - 1;
-  const bool lean_io = (!fwd || inv || dst_mode == DST_WORK) && (fwd || src_mode != SRC_F64) &&
-                       (!row || (al16(src) && al16(dst) && al16(ps.f64)));
-  const bool lean = sizeof(Real) == 4 && E <= 1 && pass_family(ax.kind) <= 2 && lean::length_ok(M) && lean_io;
+  // (lean_pass.cuh) where it has one, else the looped pass (loop_pass.cuh) where it has one, else 4
+  const bool fp32 = sizeof(Real) == 4;
+  int E = fp32 ? ax.slots32 : ax.slots64;
+  const bool deflt = fp32 ? E <= 1 : ax.loop64;
+  const bool quad = quad_io(p, ps, fp32);
+  const bool lean = fp32 && deflt && pass_family(ax.kind) <= 2 && lean::length_ok(M) && quad;
   const int lv = E == 1 ? 1 : 0;
+  // unrefined FP32 plans return the transforms' own rounding (1e-7): their bits stay those of the
+  // general pass at the lengths without a compile-time one
+  const bool unrefined = fp32 && p->precision == PC_PREC_FP32;
+  bool all = true;   // an axis without a looped pass (odd M, vertex kinds): the general passes on all
+  for (int a = 0; a < p->dim; ++a) all = all && p->ax[a].loop_nst > 0;
+  if (deflt && !lean && quad && all && !unrefined) {
+    // lines per tile: as many as the slots allow; a problem alone takes fewer where the GPU would
+    // not be full (the lines do not depend on it)
+    const int slots = fp32 ? kLoopSlots : kLoopSlots / 2;
+    int L = axis == p->dim - 1 ? 1 : 4;   // column tiles: four lines fill half a sector in FP32, one in FP64
+    while (L < 32 && 2 * L * M <= slots) L *= 2;
+    if (batch_threads <= 0) {
+      const long long lines = p->ncells / ax.n;
+      while (L > 4 && lines / L < 2 * 152) L /= 2;
+      while (L > 1 && lines / L < 152) L /= 2;   // few long lines (1024 x 96 in FP64: 152 us at four, start 86)
+    }
+    while (L > 1 && loop::tile_smem<Real>(M, L) > 160 * 1024) L /= 2;
+    tiles = fill_loop<Real>(p, ps, A, L);
+    threads = loop::kThreads;
+    smem = loop::tile_smem<Real>(M, L);
+    return PC_OK;
+  }
+  fill_pass<Real>(p, ps, A);
   if (E <= 1) E = 4;
   // threads per line: a power of two with at most E slots per thread; the kernel instance is
   // the smallest power of two >= M / tpl. A line must fit one CTA: longer lines take more
@@ -165,48 +317,15 @@ pc_status build_pass(const Plan *p, const PassSpec &ps, PassArgs<Real> &A, long 
       Ns *= si.R;
     }
   }
-  A.tw = (const T *)(sizeof(Real) == 8 ? (const void *)ax.tw64 : (const void *)ax.tw32);
-  A.dim = p->dim;
-  int stride = 1;
-  for (int b = 0; b < p->dim; ++b) A.shape[b] = (int)p->n[b];
-  for (int b = axis + 1; b < p->dim; ++b) stride *= (int)p->n[b];
-  A.stride = stride;
-  const int last = p->dim - 1;
-  A.col = axis != last;
-  A.do_fwd = fwd;
-  A.do_div = div;
-  A.do_inv = inv;
-  for (int b = 0; b < p->dim; ++b)
-    A.lam[b] = (const Real *)(sizeof(Real) == 8 ? (const void *)p->ax[b].lam64 : (const void *)p->ax[b].lam32);
-  A.singular = p->singular;
-  A.src_mode = src_mode;
-  A.src = src;
-  A.dst_mode = dst_mode;
-  A.dst = dst;
-  A.out_scale = (Real)inv_scale(ax.M);
-  A.f64 = ps.f64;
-  A.gate = ps.gate;
-  A.chunk = ps.chunk > 1 ? ps.chunk : 1;
   if (lean) {
     // compile-time tile: L lines of T = M / E threads each, 256 threads
-    const int L = lean::lines_of(M, lv);
-    if (A.col) {
-      const long long outer = p->ncells / ((long long)stride * ax.n);
-      A.inner = stride;
-      A.tiles_per_outer = (stride + L - 1) / L;
-      tiles = outer * A.tiles_per_outer;
-    } else {
-      const long long lines = p->ncells / ax.n;
-      A.lines = (int)lines;
-      tiles = (lines + L - 1) / L;
-    }
-    A.L = L;
+    tiles = fill_tiles<Real>(p, A, lean::lines_of(M, lv));
     A.lean = lean::lean_id(M, pass_family(ax.kind));
     threads = lean::kThreads;
-    A.ntiles = (int)tiles;
     smem = lean::smem_of(M, lv);
     return PC_OK;
   }
+  const int stride = A.stride;
   const int max_threads = batch_threads > 0 ? batch_threads : 256;
   const int max_lines = max_threads / tpl > 0 ? max_threads / tpl : 1;
   const int budget = 8192;          // complex slots per tile (two buffers: 2 x 64 KB in FP32)
@@ -243,7 +362,7 @@ pc_status build_pass(const Plan *p, const PassSpec &ps, PassArgs<Real> &A, long 
     return fail(PC_ERR_UNSUPPORTED, "axis %d: tile of %d x %d too large", axis, L, M);
   if (batch_threads > 0 && emax > kBatchPassEmax)
     return fail(PC_ERR_UNSUPPORTED, "axis %d: %d slots per thread exceed the batched kernel", axis, emax);
-  smem = 2 * (size_t)L * M * sizeof(T) + (size_t)L * (sizeof(Real) + 2 * sizeof(int));
+  smem = 2 * (size_t)L * M * sizeof(typename Cplx<Real>::T) + (size_t)L * (sizeof(Real) + 2 * sizeof(int));
   return PC_OK;
 }
 
@@ -258,6 +377,11 @@ static pc_status launch_pass(Plan *p, const PassSpec &ps, cudaStream_t st) {
   size_t smem;
   PC_TRY(build_pass<Real>(p, ps, A, tiles, threads, smem, 0));
   tiles = (tiles + A.chunk - 1) / A.chunk;   // CTAs
+  if (A.loop) {
+    PC_TRY(launch_loop(A, nullptr, nullptr, (unsigned)tiles, smem, st));
+    count_launch(p);
+    return PC_OK;
+  }
   if constexpr (sizeof(Real) == 4) {
     if (A.lean) {
       PC_TRY(launch_lean(A.lean, A, nullptr, nullptr, (unsigned)tiles, threads, smem, st));
@@ -280,14 +404,17 @@ static pc_status launch_pass(Plan *p, const PassSpec &ps, cudaStream_t st) {
 }
 
 // Kernel attributes set once per device, before any stream capture.
+constexpr int kPassSmem = 200 * 1024;   // dynamic shared memory of any pass
 pc_status prepare_kernels() {
-  const int lim = 200 * 1024;
+  const int lim = kPassSmem;
   PC_TRY(prepare_pass_f32_family0(lim));
   PC_TRY(prepare_pass_f32_family1(lim));
   PC_TRY(prepare_pass_f32_family2(lim));
   PC_TRY(prepare_pass_vertex(lim));
   PC_TRY(prepare_batched_f32(lim));
   PC_TRY(prepare_lean(lim));
+  PC_TRY(prepare_loop(lim));
+  PC_TRY(prepare_resident());
   PC_TRY((prepare_axis_pass_spec<double, -1, false>(lim)));
   return PC_OK;
 }
@@ -321,6 +448,103 @@ static pc_status solve_real(Plan *p, int src_mode, const void *src, int dst_mode
   if (p->dim < 2) return fail(PC_ERR_UNSUPPORTED, "dim 1");
   for (const PassSpec &ps : solve_pass_specs(p, sizeof(Real) == 4, src_mode, src, dst_mode, dst, f64, gate, chunk))
     PC_TRY(launch_pass<Real>(p, ps, st));
+  return PC_OK;
+}
+
+// Slots [first, end) of an axis's table that the wrappers of its family read.
+static void tables_of(const AxisInfo &ax, int &first, int &end) {
+  const int fam = pass_family(ax.kind), M = ax.M;
+  first = fam == 2 ? tw_dct4pre(M) : tw_rdft(M);
+  end = fam == 0 ? tw_quarter(M) : fam == 1 ? tw_dct4pre(M) : tw_total(M);
+}
+
+// Largest grid of the cooperative solve: what the SMs' shared memory holds (1024^2: 135 us against
+// 258 by launches); the fit itself is checked for each plan.
+constexpr long long kResidentCells = 1LL << 20;
+
+pc_status solve_resident(Plan *p, const double *s64, const float2 *s2, double *pout, int sweeps, bool adaptive,
+                         float tol, const GridDev &g, cudaStream_t st, bool &taken) {
+  taken = false;
+  if (p->ncells > kResidentCells || sweeps > kMaxRefine) return PC_OK;
+  for (int a = 0; a < p->dim; ++a) {
+    if (p->ax[a].slots32 != 0 || p->ax[a].loop_nst == 0) return PC_OK;
+    if (p->precision == PC_PREC_FP32 && !lean::length_ok(p->ax[a].M)) return PC_OK;   // see build_pass
+  }
+  const void *rs = s2 ? (const void *)s2 : (const void *)s64;
+  if (!aligned16(rs) || !aligned16(pout)) return PC_OK;
+  static const int sms = [] {
+    int dev = 0, n = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    return n;
+  }();
+  const int np = 2 * p->dim - 1, last = p->dim - 1;
+  ResidentArgs R;
+  memset(&R, 0, sizeof(R));
+  const std::vector<PassSpec> specs = solve_pass_specs(p, true, SRC_F32, rs, DST_PAIR_SET, p->p2);
+  // the tables behind the tiles: per axis the wrappers' factors its family reads, the stage twiddles
+  // and, on the dividing pass, the eigenvalues
+  int slots = 0, at[3][3];
+  for (int k = 0; k < p->dim; ++k) {
+    const AxisInfo &ax = p->ax[specs[k].axis];
+    int *t = at[specs[k].axis], first, end;
+    tables_of(ax, first, end);
+    t[0] = slots - first;
+    slots += end - first;
+    t[1] = slots;
+    slots += loop_twiddles(ax);
+    t[2] = 2 * slots;
+    if (specs[k].div) slots += (ax.n + 1) / 2;
+  }
+  slots = (slots + 1) & ~1;
+  // lines per tile: as few as give every SM at most one tile, and fewer again where
+  // the buffers would not leave room for the own rows
+  size_t smem = 0;
+  bool fits = false;
+  for (int cap = 2 * kLoopSlots; cap >= kLoopSlots / 2 && !fits; cap /= 2) {
+    long long most = 0;
+    size_t tiles_smem = 0;
+    for (int k = 0; k < np; ++k) {
+      const int M = p->ax[specs[k].axis].M;
+      const long long lines = p->ncells / p->ax[specs[k].axis].n;
+      int L = 1;
+      while ((lines + L - 1) / L > sms && 2 * L * M <= cap) L *= 2;
+      const long long tiles = fill_loop<float>(p, specs[k], R.pass[k], L);
+      most = tiles > most ? tiles : most;
+      const size_t b = loop::tile_smem<float>(M, L);
+      tiles_smem = b > tiles_smem ? b : tiles_smem;
+    }
+    R.grid = (int)(most < sms ? most : sms);
+    R.row_tiles = (R.pass[0].ntiles + R.grid - 1) / R.grid;
+    R.tables_at = (int)((tiles_smem + 15) / 16 * 2);
+    R.own_at = R.tables_at + slots;
+    smem = (size_t)R.own_at * sizeof(float2) + (size_t)R.row_tiles * R.pass[0].L * p->ax[last].n * 4 * sizeof(float);
+    fits = smem <= (size_t)kResidentSmem;
+  }
+  if (!fits) return PC_OK;
+  for (int k = 0; k < np; ++k) {
+    PassArgs<float> &A = R.pass[k];
+    const AxisInfo &ax = p->ax[specs[k].axis];
+    const int *t = at[specs[k].axis];
+    tables_of(ax, A.tw_first, A.tw_last);
+    A.tw_at = t[0];
+    A.st_at = t[1];
+    A.st_count = loop_twiddles(ax);
+    A.lam_at = t[2];
+  }
+  R.g = g;
+  R.s = rs;
+  R.p2 = p->p2;
+  R.f64 = pout;
+  R.st = p->dstats;
+  R.bar = p->dstats->bar;
+  R.sweeps = sweeps;
+  R.adaptive = adaptive;
+  R.singular = p->singular;
+  R.tol = tol;
+  PC_TRY(launch_resident(R, p->dim, s2 != nullptr, smem, st));
+  count_launch(p);
+  taken = true;
   return PC_OK;
 }
 

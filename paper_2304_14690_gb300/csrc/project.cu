@@ -1011,7 +1011,7 @@ static dim3 vertex_grid_dims(int dim, const int *shape, int threads) {
               dim == 3 ? (unsigned)shape[0] : 1u);
 }
 
-static GridDev grid_dev(const Plan *p);
+
 
 static VertexGrid vertex_grid(const Plan *p) {
   VertexGrid V{};
@@ -1237,7 +1237,7 @@ void batch_problem_fill(const Plan *p, const pc_project_args &a, BatchProblem &q
 }
 
 // ----------------------------------------------------------------------------- host
-static GridDev grid_dev(const Plan *p) {
+GridDev grid_dev(const Plan *p) {
   GridDev g{};
   g.dim = p->dim;
   g.mask = (p->rhs_mask_on && !p->vertex) ? p->rhs_mask : nullptr;   // vertex plans mask their unknowns
@@ -1377,11 +1377,16 @@ static pc_status solve_grid(Plan *p, const double *s64, double *pout, bool want_
     auto step = [&](int k) { return RefineStep{k, adaptive ? 1 : 0, tol, chunk(k)}; };
     auto gate = [&](int j) { return adaptive ? RefineGate{p->dstats, j, tol} : RefineGate{nullptr, 0, 0.0f}; };
     const bool norm = want_final_residual;
+    // the whole refined solve in one cooperative kernel where it fits; statistics need the residuals'
+    // L2 norms and take the launches below (the same bits)
+    bool resident = false;
+    if (!norm) PC_TRY(solve_resident(p, s64, s2, pout, sweeps, adaptive, tol, g, st, resident));
     double *first_out = (sweeps == 0 || adaptive) ? pout : nullptr;
-    if (s32) PC_TRY(solve_fp32_grid(p, SRC_F32_, s32, DST_PAIR_SET_, p->p2, st, first_out));
+    if (resident) ;
+    else if (s32) PC_TRY(solve_fp32_grid(p, SRC_F32_, s32, DST_PAIR_SET_, p->p2, st, first_out));
     else PC_TRY(solve_fp32_grid(p, SRC_F64_, s64, DST_PAIR_SET_, p->p2, st, first_out));
     prof_mark(p, st, 3);
-    for (int it = 0; it < sweeps; ++it) {
+    for (int it = 0; it < sweeps && !resident; ++it) {
       float *r32 = reinterpret_cast<float *>(p->work64);   // work64 is free in mixed mode
       if (s2)
         launch_residual(p->singular, true, norm, st, g, s2, (const float2 *)p->p2, r32, p->dstats,
@@ -1718,9 +1723,11 @@ static pc_status vertex_solve(Plan *p, const double *s, double *p_out, pc_stats 
   if (hp) dp = p->stage_p;
   prof_begin(p, st);
   PC_CUDA_TRY(cudaMemsetAsync(p->dstats, 0, sizeof(DevStats), st));
-  launch_pdl(sum_kernel, grid_for(nc, kFlatPerBlock), kFlatThreads, 0, st, nc, ds, p->dstats, p->partials,
-             p->counters, trap_weights(p));
-  count_launch(p);
+  if (p->singular || stats) {   // the sums: the mean of a zero-mode problem, and the statistics
+    launch_pdl(sum_kernel, grid_for(nc, kFlatPerBlock), kFlatThreads, 0, st, nc, ds, p->dstats, p->partials,
+               p->counters, trap_weights(p));
+    count_launch(p);
+  }
   prof_mark(p, st, 2);
   PC_TRY(solve_grid(p, ds, dp, stats != nullptr, st));
   PC_CUDA_TRY(cudaGetLastError());
@@ -1740,9 +1747,11 @@ static pc_status solve_impl(Plan *p, const double *s, double *p_out, pc_stats *s
   if (hp) dp = p->stage_p;
   prof_begin(p, st);
   PC_CUDA_TRY(cudaMemsetAsync(p->dstats, 0, sizeof(DevStats), st));
-  launch_pdl(sum_kernel, grid_for(nc, kFlatPerBlock), kFlatThreads, 0, st, nc, ds, p->dstats, p->partials, p->counters,
-             TrapWeights{});
-  count_launch(p);
+  if (p->singular || stats) {   // the sums: the mean of a zero-mode problem, and the statistics
+    launch_pdl(sum_kernel, grid_for(nc, kFlatPerBlock), kFlatThreads, 0, st, nc, ds, p->dstats, p->partials, p->counters,
+               TrapWeights{});
+    count_launch(p);
+  }
   prof_mark(p, st, 2);
   PC_TRY(solve_grid(p, ds, dp, stats != nullptr, st));
   if (hp) PC_CUDA_TRY(cudaMemcpyAsync(p_out, dp, nc * sizeof(double), cudaMemcpyDeviceToHost, st));

@@ -25,6 +25,9 @@ static bool valid_ctas(int c) { return c == 1 || c == 2 || c == 4 || c == 8; }
 // One solve of the plan's transform precision from s64 into the staging buffer.
 static pc_status run_solve(Plan *p, bool fp64, cudaStream_t st) {
   if (fp64) return solve_fp64_grid(p, p->s64, p->stage_p, st);
+  bool taken = false;   // grids of the cooperative solve: one launch under the default schedule
+  PC_TRY(solve_resident(p, p->s64, nullptr, p->stage_p, 0, false, 0.0f, grid_dev(p), st, taken));
+  if (taken) return PC_OK;
   return solve_fp32_grid(p, SRC_F64, p->s64, DST_F64_SET, p->stage_p, st);
 }
 
@@ -56,7 +59,8 @@ static pc_status autotune(Plan *p, cudaStream_t st, double *best_out) {
   pc_status status = PC_OK;
   float best = 0.0f;
   const int reps = p->ncells > (1 << 22) ? 3 : (p->ncells > (1 << 18) ? 10 : 30);
-  if (cudaMemsetAsync(p->s64, 0, p->ncells * sizeof(double), st) != cudaSuccess)
+  if (cudaMemsetAsync(p->s64, 0, p->ncells * sizeof(double), st) != cudaSuccess ||
+      cudaMemsetAsync(p->dstats, 0, sizeof(DevStats), st) != cudaSuccess)
     status = fail(PC_ERR_CUDA, "cudaMemsetAsync failed");
   if (status == PC_OK) status = time_solve(p, fp64, st, e0, e1, reps, best);
   for (int round = 0; round < 2 && status == PC_OK; ++round) {
@@ -66,15 +70,18 @@ static pc_status autotune(Plan *p, cudaStream_t st, double *best_out) {
       for (int knob = 0; knob < 2; ++knob) {
         int &s = knob == 0 ? slots_ref(p, a, fp64) : ctas_ref(p, a, fp64);
         for (int cand : {0, 1, 2, 4, 8, 16}) {
-          if (cand == s || (knob == 0 ? !valid_slots(cand, fp64) : !valid_ctas(cand))) continue;
+          if ((cand == s && !(fp64 && knob == 0 && p->ax[a].loop64)) || (knob == 0 ? !valid_slots(cand, fp64) : !valid_ctas(cand))) continue;
           const int keep = s;
+          const bool keep_loop = p->ax[a].loop64;
           s = cand;
+          if (fp64) p->ax[a].loop64 = false;
           float t = 0.0f;
           const pc_status r = time_solve(p, fp64, st, e0, e1, reps, t);
           if (r != PC_OK) {
             // a schedule the kernels cannot run (a tile too large): not a candidate
             cudaGetLastError();
             s = keep;
+            p->ax[a].loop64 = keep_loop;
             continue;
           }
           if (t < 0.98f * best) {
@@ -82,6 +89,7 @@ static pc_status autotune(Plan *p, cudaStream_t st, double *best_out) {
             changed = true;
           } else {
             s = keep;
+            p->ax[a].loop64 = keep_loop;
           }
         }
       }
@@ -104,6 +112,7 @@ extern "C" pc_status pc_plan_set_transform_slots(pc_plan *plan, int axis, pc_pre
   if (!pc::valid_slots(slots, precision == PC_PREC_FP64))
     return pc::fail(PC_ERR_INVALID_ARG, "slots must be 2, 4, 8 or 16, or 0 or 1 for FP32 (got %d)", slots);
   pc::slots_ref(p, axis, precision == PC_PREC_FP64) = slots;
+  if (precision == PC_PREC_FP64) p->ax[axis].loop64 = false;
   pc::plan_drop_graphs(p);
   return PC_OK;
 }
