@@ -117,6 +117,19 @@ __device__ __forceinline__ DF2 second_difference2(DF2 pl, DF2 pc, DF2 pr, DF ih2
   return DF2{p, f2_fma(t.lo, hh, e)};
 }
 
+__device__ __forceinline__ F2 f2_neg(F2 a) { return F2{a.v ^ 0x8000000080000000ULL}; }
+__device__ __forceinline__ DF2 df2_neg(DF2 a) { return DF2{f2_neg(a.hi), f2_neg(a.lo)}; }
+// The ghost of an edge value: itself (Neumann) or its negative (Dirichlet).
+__device__ __forceinline__ DF2 ghost(int kind, DF2 v) { return kind ? df2_neg(v) : v; }
+// (last of a, first of b): the pair between two neighbouring pairs.
+__device__ __forceinline__ F2 f2_mid(F2 a, F2 b) { return F2{(a.v >> 32) | (b.v << 32)}; }
+__device__ __forceinline__ DF2 df2_mid(DF2 a, DF2 b) { return DF2{f2_mid(a.hi, b.hi), f2_mid(a.lo, b.lo)}; }
+__device__ __forceinline__ float max_abs(float m, F2 v) {
+  float x, y;
+  f2_unpack(v, x, y);
+  return fmaxf(m, fmaxf(fabsf(x), fabsf(y)));
+}
+
 // A stored value as a double-float pair: FP64 values are split exactly as split_f64 does, pairs
 // are taken as they are.
 __device__ __forceinline__ DF to_df(double v) { return df_of(v); }

@@ -237,7 +237,7 @@ struct Plan {
   uint8_t *ntype = nullptr;    // [N]
 
   // Workspace (allocated once; pc_project allocates nothing).
-  double *U64[3] = {nullptr, nullptr, nullptr};  // face fluxes
+  double *U64[3] = {nullptr, nullptr, nullptr};  // face fluxes (FP64, or float2 pairs: mixed and FP32 plans)
   double *s64 = nullptr;       // source
   double *p64 = nullptr;       // pressure (refined iterate)
   double *work64 = nullptr;    // FP64 transform workspace (cells)
@@ -401,6 +401,7 @@ struct BatchProblem {
   int dim, vdtype, N, ncells, K, Kg, singular, gmode;
   int kmax;            // refinement sweeps at most; under the stopping rule when tol > 0
   float tol;           // the rule's tolerance (<= 0: a fixed sweep count)
+  int pair_blocks;     // blocks of the residual (two cells per thread)
   const void *u, *f;
   void *uo, *fo;
   double *p;

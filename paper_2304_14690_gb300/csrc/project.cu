@@ -15,7 +15,9 @@
 #include <cmath>
 #include <cstdio>
 #include <cstddef>
+#include <cstdint>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "dfloat.cuh"
@@ -231,7 +233,7 @@ struct PairSrc {
 };
 
 template <int KC, typename Src>
-__device__ __forceinline__ double transfer_mixed_row(int r, int rows, int Kr, const int32_t *__restrict__ col,
+__device__ __forceinline__ float2 transfer_mixed_row(int r, int rows, int Kr, const int32_t *__restrict__ col,
                                                      const float2 *__restrict__ w2, Src src) {
   const int K = KC > 0 ? KC : Kr;
   DF s{0.f, 0.f};
@@ -252,19 +254,22 @@ __device__ __forceinline__ double transfer_mixed_row(int r, int rows, int Kr, co
       df_acc(s, __ldcs(w2 + at), src(__ldcs(col + at)));
     }
   }
-  return df_value(s);
+  // the flux stays a pair, renormalised without error (TwoSum): the divergence takes pairs
+  float hi, lo;
+  two_sum(s.hi, s.lo, hi, lo);
+  return make_float2(hi, lo);
 }
 template <int KC, typename Src>
 __device__ __forceinline__ void transfer_mixed_kernel_body(const VBlock &vb, int rows, int Kr, const int32_t *__restrict__ col,
                                       const float2 *__restrict__ w2, Src src,
-                                      double *__restrict__ U) {
+                                      float2 *__restrict__ U) {
   int r = vb.x * blockDim.x + threadIdx.x;
   if (r >= rows) return;
   U[r] = transfer_mixed_row<KC>(r, rows, Kr, col, w2, src);
 }
 template <int KC, typename Src>
 __global__ void transfer_mixed_kernel(int rows, int Kr, const int32_t *__restrict__ col,
-                                      const float2 *__restrict__ w2, Src src, double *__restrict__ U) {
+                                      const float2 *__restrict__ w2, Src src, float2 *__restrict__ U) {
   pdl_enter();
   transfer_mixed_kernel_body<KC>(hw_block(), rows, Kr, col, w2, src, U);
 }
@@ -307,69 +312,71 @@ __device__ __forceinline__ VBlock tile_block(const GridDev &g, unsigned b) {
 }
 
 // ----------------------------------------------------------------------------- divergence
-// s = D_h U / (beta dt) (FP64; as an FP32 pair in double-float arithmetic on the mixed path),
-// its FP32 copy; want_sums 1: sum(s) and the mean, 2: also sum(s^2) (statistics).
-template <int DIM>
-__device__ __forceinline__ void divergence_body(unsigned b, const GridDev &g, const double *U0, const double *U1,
-                                                const double *U2, double inv_bdt, double *s, float2 *s2, float *s32,
-                                                DevStats *stats, double *partials, unsigned int *counter,
-                                                int want_sums, double inv_ncells) {
+// s = D_h U / (beta dt), from FP64 faces (FP64 path) or from faces kept as FP32 pairs (mixed path: in
+// double-float arithmetic, FP32 operations with error-free transformations, about 48 bits; the FP64
+// pipe runs at a small fraction of the FP32 rate on this GPU). The mixed source is stored as a pair
+// and as its FP32 copy; want_sums 1: sum(s) and the mean, 2: also sum(s^2) (statistics).
+__device__ __forceinline__ double face_diff(double hi, double lo) { return hi - lo; }
+__device__ __forceinline__ DF face_diff(float2 hi, float2 lo) { return df_sub(DF{hi.x, hi.y}, DF{lo.x, lo.y}); }
+template <int DIM, typename UT>
+__device__ __forceinline__ void divergence_body(unsigned b, const GridDev &g, const UT *U0, const UT *U1, const UT *U2,
+                                                double inv_bdt, double *s, float2 *s2, float *s32, DevStats *stats,
+                                                double *partials, unsigned int *counter, int want_sums,
+                                                double inv_ncells) {
   int x, row0;
   tile_pos(g, b, x, row0);
-  const double *U[3] = {U0, U1, U2};
-  double c[DIM];
-#pragma unroll
-  for (int a = 0; a < DIM; ++a) c[a] = g.inv_h[a] * inv_bdt;
+  const UT *U[3] = {U0, U1, U2};
   double sum = 0.0, sum2 = 0.0;
-  if (s2 && x < g.n[DIM - 1]) {
-    // mixed path: the source is kept as an FP32 pair, so it is formed in double-float arithmetic
-    // (FP32 operations with error-free transformations, about 48 bits) from the FP64 faces: the
-    // FP64 pipe runs at a small fraction of the FP32 rate on this GPU
-    DF cd[DIM];
-#pragma unroll
-    for (int a = 0; a < DIM; ++a) cd[a] = df_of(c[a]);
-    DF sd{0.0f, 0.0f}, sd2{0.0f, 0.0f};
+  if (x < g.n[DIM - 1]) {
     const int rend = min(row0 + g.cr, g.rows);
-    for (int row = row0; row < rend; ++row) {
-      int i[3];
-      cell_at<DIM>(g, row, x, i);
-      DF v{0.0f, 0.0f};
+    if constexpr (sizeof(UT) == sizeof(double) && std::is_same<UT, double>::value) {
+      double c[DIM];
 #pragma unroll
-      for (int a = 0; a < DIM; ++a) {
-        int hi = i[a] + 1;
-        if (g.periodic[a] && hi == g.n[a]) hi = 0;
-        const DF d = df_sub(df_of(U[a][face_index(g, a, i, hi)]), df_of(U[a][face_index(g, a, i, i[a])]));
-        v = (a == 0) ? df_mul(d, cd[0]) : df_add(v, df_mul(d, cd[a]));
-      }
-      const int ci = cell_index(g, i);
-      if (g.mask && !g.mask[ci]) v = DF{0.0f, 0.0f};   // outside the flow domain (RHS mask)
-      s2[ci] = make_float2(v.hi, v.lo);
-      if (s32) s32[ci] = v.hi;   // FP32 copy read by the first FP32 transform pass
-      if (want_sums) sd = df_add(sd, v);
-      if (want_sums > 1) sd2 = df_add(sd2, df_mul(v, v));
-    }
-    sum = f2d_bits(sd.hi) + f2d_bits(sd.lo);
-    sum2 = f2d_bits(sd2.hi) + f2d_bits(sd2.lo);
-  } else if (x < g.n[DIM - 1]) {
-    const int rend = min(row0 + g.cr, g.rows);
-    for (int row = row0; row < rend; ++row) {
-      int i[3];
-      cell_at<DIM>(g, row, x, i);
-      double v = 0.0;
+      for (int a = 0; a < DIM; ++a) c[a] = g.inv_h[a] * inv_bdt;
+      for (int row = row0; row < rend; ++row) {
+        int i[3];
+        cell_at<DIM>(g, row, x, i);
+        double v = 0.0;
 #pragma unroll
-      for (int a = 0; a < DIM; ++a) {
-        int hi = i[a] + 1;
-        if (g.periodic[a] && hi == g.n[a]) hi = 0;
-        const double d = U[a][face_index(g, a, i, hi)] - U[a][face_index(g, a, i, i[a])];
-        v = (a == 0) ? d * c[0] : fma(d, c[a], v);
+        for (int a = 0; a < DIM; ++a) {
+          int hi = i[a] + 1;
+          if (g.periodic[a] && hi == g.n[a]) hi = 0;
+          const double d = face_diff(U[a][face_index(g, a, i, hi)], U[a][face_index(g, a, i, i[a])]);
+          v = (a == 0) ? d * c[0] : fma(d, c[a], v);
+        }
+        const int ci = cell_index(g, i);
+        if (g.mask && !g.mask[ci]) v = 0.0;   // outside the flow domain (RHS mask)
+        s[ci] = v;
+        if (want_sums) sum += v;
+        if (want_sums > 1) sum2 = fma(v, v, sum2);
       }
-      const int ci = cell_index(g, i);
-      if (g.mask && !g.mask[ci]) v = 0.0;   // outside the flow domain (RHS mask)
-      if (s2) s2[ci] = as_pair(v);     // the refinement keeps s as a (hi, lo) pair
-      else s[ci] = v;
-      if (s32) s32[ci] = d2f_rz_bits(v);   // FP32 copy read by the first FP32 transform pass
-      if (want_sums) sum += v;
-      if (want_sums > 1) sum2 = fma(v, v, sum2);
+    } else {
+      DF cd[DIM];
+#pragma unroll
+      for (int a = 0; a < DIM; ++a) cd[a] = df_of(g.inv_h[a] * inv_bdt);
+      DF sd{0.0f, 0.0f}, sd2{0.0f, 0.0f};
+      for (int row = row0; row < rend; ++row) {
+        int i[3];
+        cell_at<DIM>(g, row, x, i);
+        DF v{0.0f, 0.0f};
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) {
+          int hi = i[a] + 1;
+          if (g.periodic[a] && hi == g.n[a]) hi = 0;
+          const DF d = face_diff(U[a][face_index(g, a, i, hi)], U[a][face_index(g, a, i, i[a])]);
+          v = (a == 0) ? df_mul(d, cd[0]) : df_add(v, df_mul(d, cd[a]));
+        }
+        const int ci = cell_index(g, i);
+        if (g.mask && !g.mask[ci]) v = DF{0.0f, 0.0f};   // outside the flow domain (RHS mask)
+        s2[ci] = make_float2(v.hi, v.lo);
+        if (s32) s32[ci] = v.hi;   // FP32 copy read by the first FP32 transform pass
+        if (want_sums) sd = df_add(sd, v);
+        if (want_sums > 1) sd2 = df_add(sd2, df_mul(v, v));
+      }
+      if (want_sums) {
+        sum = f2d_bits(sd.hi) + f2d_bits(sd.lo);
+        sum2 = f2d_bits(sd2.hi) + f2d_bits(sd2.lo);
+      }
     }
   }
   if (want_sums) {
@@ -379,13 +386,13 @@ __device__ __forceinline__ void divergence_body(unsigned b, const GridDev &g, co
   }
 }
 
-template <int DIM>
-__global__ void divergence_kernel(GridDev g, const double *U0, const double *U1, const double *U2,
+template <int DIM, typename UT>
+__global__ void divergence_kernel(GridDev g, const UT *U0, const UT *U1, const UT *U2,
                                   double inv_bdt, double *s, float2 *s2, float *s32, DevStats *stats,
                                   double *partials, unsigned int *counter, int want_sums, double inv_ncells) {
   pdl_enter();
-  divergence_body<DIM>(blockIdx.x, g, U0, U1, U2, inv_bdt, s, s2, s32, stats, partials, counter, want_sums,
-                       inv_ncells);
+  divergence_body<DIM, UT>(blockIdx.x, g, U0, U1, U2, inv_bdt, s, s2, s32, stats, partials, counter, want_sums,
+                           inv_ncells);
 }
 
 // Direct divergence (PC_DIV_WLS_DIRECT): s = (1/(beta dt)) sum_a sum_k D_a,k u~_a,k at every
@@ -630,6 +637,121 @@ __global__ void residual_kernel(GridDev g, const SV *__restrict__ s, const PV *_
   residual_record(rs, rmx, smx, stats);
 }
 
+// The residual of two neighbouring cells per thread and row (packed FP32 operations, 16-byte
+// accesses; n of the last axis is even on every cell grid), the thread walking its rows with the
+// rows above and below kept in registers: r and the rule's max norms, cell for cell with the bits of
+// residual_body, which the launches with L2 norms (statistics) and vertex grids keep. The kernel
+// is bound by instructions: about 75 per cell instead of 190.
+__device__ __forceinline__ DF2 load_two(const float2 *p) {
+  const float4 v = *reinterpret_cast<const float4 *>(p);
+  return DF2{f2_pack(v.x, v.z), f2_pack(v.y, v.w)};
+}
+__device__ __forceinline__ DF2 load_two(const double *p) {
+  const double2 v = *reinterpret_cast<const double2 *>(p);
+  return df2_of(df_of(v.x), df_of(v.y));
+}
+// Blocks of 2^bits threads along the last axis (pairs of cells) by 2^(8 - bits) thread rows of
+// kPairRows rows each.
+constexpr int kPairRows = 4;
+__host__ __device__ inline int pair_bits(const GridDev &g) { return g.tw_bits - 1; }
+__host__ __device__ inline int pair_gx(const GridDev &g) {
+  const int w = 2 << pair_bits(g), nl = g.n[g.dim - 1];
+  return (nl + w - 1) / w;
+}
+static int pair_blocks(const GridDev &g) {
+  const int rpb = kPairRows << (8 - pair_bits(g));
+  return pair_gx(g) * ((g.rows + rpb - 1) / rpb);
+}
+template <int DIM, bool SINGULAR, typename SV>
+__device__ __forceinline__ void residual_pair_body(unsigned b, const GridDev &g, const SV *__restrict__ s,
+                                                   const float2 *__restrict__ p, float *__restrict__ r,
+                                                   const DevStats *stats, const RefineStep &rs, float &rmx, float &smx) {
+  const int bits = pair_bits(g), gx = pair_gx(g), t = threadIdx.x, nl = g.n[DIM - 1];
+  const int by = (int)(b / (unsigned)gx), bx = (int)b - by * gx;
+  const int x = 2 * ((bx << bits) + (t & ((1 << bits) - 1)));
+  const int row0 = ((by << (8 - bits)) + (t >> bits)) * kPairRows;
+  const int rend = min(row0 + kPairRows, g.rows);
+  if (x >= nl || row0 >= rend) return;
+  DF2 mean{F2{0ULL}, F2{0ULL}};
+  if (SINGULAR) {
+    const DF m = df_of(stats->mean_s);
+    mean = df2_of(m, m);
+  }
+  constexpr int w = DIM - 2;   // the axis the thread walks along
+  const bool per = g.periodic[w];
+  const int xl = x > 0 ? -1 : nl - 1, xr = x + 2 < nl ? 2 : 2 - nl;   // of x
+  DF2 pc, pu, pd;
+  bool have = false;           // pu and pc carried over from the row before
+  for (int row = row0; row < rend; ++row) {
+    int i[3];
+    cell_at<DIM>(g, row, x, i);
+    const int c = cell_index(g, i);
+    if (!have) {
+      pc = load_two(p + c);
+      if (i[w] > 0 || per) pu = load_two(p + (i[w] > 0 ? c - nl : c + (g.n[w] - 1) * nl));
+      else pu = ghost(g.lo_kind[w], pc);
+    }
+    const bool inside = i[w] < g.n[w] - 1;
+    if (inside || per) pd = load_two(p + (inside ? c + nl : c - (g.n[w] - 1) * nl));
+    else pd = ghost(g.hi_kind[w], pc);
+    const float2 el = p[c + xl], er = p[c + xr];
+    DF2 acc;
+    if (DIM == 3) {
+      const int st = g.cs[0];
+      const bool lin = i[0] > 0, hin = i[0] < g.n[0] - 1, p0 = g.periodic[0];
+      DF2 lo, hi;
+      if (lin || p0) lo = load_two(p + (lin ? c - st : c + (g.n[0] - 1) * st));
+      else lo = ghost(g.lo_kind[0], pc);
+      if (hin || p0) hi = load_two(p + (hin ? c + st : c - (g.n[0] - 1) * st));
+      else hi = ghost(g.hi_kind[0], pc);
+      acc = second_difference2(lo, pc, hi, DF{g.ih2_hi[0], g.ih2_lo[0]});
+      acc = df2_sum(acc, second_difference2(pu, pc, pd, DF{g.ih2_hi[w], g.ih2_lo[w]}));
+    } else {
+      acc = second_difference2(pu, pc, pd, DF{g.ih2_hi[w], g.ih2_lo[w]});
+    }
+    {
+      constexpr int a = DIM - 1;
+      DF2 l = DF2{f2_pack(0.0f, el.x), f2_pack(0.0f, el.y)}, e = DF2{f2_pack(er.x, 0.0f), f2_pack(er.y, 0.0f)};
+      if (x == 0 && !g.periodic[a]) {
+        const DF2 v = ghost(g.lo_kind[a], pc);
+        l = DF2{F2{v.hi.v << 32}, F2{v.lo.v << 32}};
+      }
+      if (x + 2 >= nl && !g.periodic[a]) {
+        const DF2 v = ghost(g.hi_kind[a], pc);
+        e = DF2{F2{v.hi.v >> 32}, F2{v.lo.v >> 32}};
+      }
+      acc = df2_sum(acc, second_difference2(df2_mid(l, pc), pc, df2_mid(pc, e), DF{g.ih2_hi[a], g.ih2_lo[a]}));
+    }
+    DF2 sv = load_two(s + c);
+    if (rs.rule && rs.k == 0) smx = max_abs(smx, sv.hi);
+    if (SINGULAR) sv = df2_diff(sv, mean);
+    const DF2 v = df2_diff(sv, acc);
+    const F2 h = f2_add(v.hi, v.lo);
+    float2 out;
+    f2_unpack(h, out.x, out.y);
+    *reinterpret_cast<float2 *>(r + c) = out;
+    if (rs.rule) rmx = fmaxf(rmx, fmaxf(fabsf(out.x), fabsf(out.y)));
+    have = inside;
+    pu = pc;
+    pc = pd;
+  }
+}
+// CTA b evaluates blocks b * rs.chunk, ... of nblk.
+template <int DIM, bool SINGULAR, typename SV>
+__global__ void __launch_bounds__(256) residual_pair_kernel(GridDev g, const SV *__restrict__ s, const float2 *__restrict__ p,
+                                                            float *__restrict__ r, DevStats *stats, RefineStep rs, int nblk) {
+  pdl_enter();
+  // as in residual_kernel
+  if (rs.rule == 1 && rs.k > 0 &&
+      (gridDim.x >= 512 ? cta_refine_stopped_before(stats, rs.k, rs.tol) : refine_stopped_before(stats, rs.k, rs.tol)))
+    return;
+  const int c = rs.chunk > 1 ? rs.chunk : 1;
+  const int b0 = blockIdx.x * c, b1 = min(b0 + c, nblk);
+  float rmx = 0.0f, smx = 0.0f;
+  for (int b = b0; b < b1; ++b) residual_pair_body<DIM, SINGULAR, SV>(b, g, s, p, r, stats, rs, rmx, smx);
+  residual_record(rs, rmx, smx, stats);
+}
+
 // ----------------------------------------------------------------------------- gauge
 // Sum of p (weighted, see TrapWeights; and the corner value); the reducing block stores the
 // gauge constant.
@@ -846,13 +968,15 @@ __global__ void gradient_mixed_kernel(int N, BlockGrid bg, const int32_t *__rest
 // ----------------------------------------------------------------------------- check
 // max over cells of |D_h (U - beta dt G_h p)|; wall faces carry no flux and no gradient. Cells
 // outside the RHS mask are skipped.
-template <int DIM>
-__global__ void div_check_kernel(GridDev g, const double *U0, const double *U1,
-                                 const double *U2, const double *p, double bdt, DevStats *stats) {
+__device__ __forceinline__ double face_value(double u) { return u; }
+__device__ __forceinline__ double face_value(float2 u) { return f2d_bits(u.x) + f2d_bits(u.y); }
+template <int DIM, typename UT>
+__global__ void div_check_kernel(GridDev g, const UT *U0, const UT *U1,
+                                 const UT *U2, const double *p, double bdt, DevStats *stats) {
   pdl_enter();
   int x, row0;
   tile_pos(g, blockIdx.x, x, row0);
-  const double *U[3] = {U0, U1, U2};
+  const UT *U[3] = {U0, U1, U2};
   double v = 0.0;
   if (x < g.n[DIM - 1]) {
     const int rend = min(row0 + g.cr, g.rows);
@@ -870,8 +994,8 @@ __global__ void div_check_kernel(GridDev g, const double *U0, const double *U1,
         neighbours(g, p, i, c, a, pc, pl, pr);
         int hi = i[a] + 1;
         if (g.periodic[a] && hi == g.n[a]) hi = 0;
-        const double Ulo = U[a][face_index(g, a, i, i[a])] - bdt * (pc - pl) * g.inv_h[a];
-        const double Uhi = U[a][face_index(g, a, i, hi)] - bdt * (pr - pc) * g.inv_h[a];
+        const double Ulo = face_value(U[a][face_index(g, a, i, i[a])]) - bdt * (pc - pl) * g.inv_h[a];
+        const double Uhi = face_value(U[a][face_index(g, a, i, hi)]) - bdt * (pr - pc) * g.inv_h[a];
         acc += (Uhi - Ulo) * g.inv_h[a];
       }
       v = fmax(v, fabs(acc));
@@ -942,7 +1066,7 @@ __global__ void ib_transfer64_kernel(int nl, const int32_t *__restrict__ list, i
 template <int KC>
 __global__ void ib_transfer_mixed_kernel(int nl, const int32_t *__restrict__ list, int rows, int Kr,
                                          const int32_t *__restrict__ col, const float2 *__restrict__ w2,
-                                         PairSrc src, double *__restrict__ U) {
+                                         PairSrc src, float2 *__restrict__ U) {
   pdl_enter();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= nl) return;
@@ -1147,7 +1271,7 @@ __global__ void batch_transfer(const BatchProblem *__restrict__ P, const int *__
   const BatchProblem &q = P[pi];
   const VBlock vb = flat_block(blockIdx.x - seg[pi], seg[pi + 1] - seg[pi]);
   transfer_mixed_kernel_body<KC>(vb, q.frows[a], q.K, q.fcol[a], q.fw2[a], PairSrc{q.u2 + (long long)a * q.N},
-                                 q.U64[a]);
+                                 reinterpret_cast<float2 *>(q.U64[a]));
 }
 
 // Cell and residual stages of a group (one dimension per group: DIM is a template parameter).
@@ -1168,18 +1292,20 @@ __global__ void batch_divergence(const BatchProblem *__restrict__ P, const int *
   const BatchProblem &q = P[pi];
   const unsigned lb = blockIdx.x - seg[pi];
   const GridDev &g = stage_grid(q.g);
-  divergence_body<DIM>(lb, g, q.U64[0], q.U64[1], q.U64[2], q.inv_bdt, nullptr, reinterpret_cast<float2 *>(q.s64),
-                       q.s32, q.ds, q.partials, q.counters, q.singular, q.inv_ncells);
+  const float2 *U[3] = {reinterpret_cast<const float2 *>(q.U64[0]), reinterpret_cast<const float2 *>(q.U64[1]),
+                        reinterpret_cast<const float2 *>(q.U64[2])};
+  divergence_body<DIM, float2>(lb, g, U[0], U[1], U[2], q.inv_bdt, nullptr, reinterpret_cast<float2 *>(q.s64), q.s32,
+                                q.ds, q.partials, q.counters, q.singular, q.inv_ncells);
 }
 
 // Residual k of every problem (k sweeps done). Problems under the stopping rule (tol > 0)
 // record the max norm of r_k and skip the launch once the rule ended their refinement. A CTA
-// evaluates kResidualChunk consecutive blocks of its problem's single-call decomposition (the
-// residual per cell and its max norm do not depend on how blocks are grouped), so a skipped
+// evaluates kResidualChunk consecutive blocks of its problem (the residual per cell and its max norm
+// do not depend on how blocks are grouped), so a skipped
 // launch costs a quarter of the CTAs.
 constexpr int kResidualChunk = 4;
 template <int DIM>
-__global__ void batch_residual(const BatchProblem *__restrict__ P, const int *__restrict__ seg, int count, int k) {
+__global__ void __launch_bounds__(256, 4) batch_residual(const BatchProblem *__restrict__ P, const int *__restrict__ seg, int count, int k) {
   pdl_enter();
   const int pi = batch_problem_of(seg, count, blockIdx.x);
   const BatchProblem &q = P[pi];
@@ -1188,11 +1314,11 @@ __global__ void batch_residual(const BatchProblem *__restrict__ P, const int *__
   if (rule && k > 0 && cta_refine_stopped_before(q.ds, k, q.tol)) return;
   const RefineStep rs{k, rule ? 2 : 0, q.tol, 1};
   const int b0 = (int)(blockIdx.x - seg[pi]) * kResidualChunk;
-  const int b1 = min(b0 + kResidualChunk, q.g.nblk);
+  const int b1 = min(b0 + kResidualChunk, q.pair_blocks);
   float rmx = 0.0f, smx = 0.0f;
   for (int b = b0; b < b1; ++b) {
-    if (q.singular) residual_body<DIM, true, true, false>(b, q.g, s2, q.p2, q.r32, q.ds, nullptr, q.partials, q.counters, rs, rmx, smx);
-    else residual_body<DIM, false, true, false>(b, q.g, s2, q.p2, q.r32, q.ds, nullptr, q.partials, q.counters, rs, rmx, smx);
+    if (q.singular) residual_pair_body<DIM, true>(b, q.g, s2, q.p2, q.r32, q.ds, rs, rmx, smx);
+    else residual_pair_body<DIM, false>(b, q.g, s2, q.p2, q.r32, q.ds, rs, rmx, smx);
   }
   residual_record(rs, rmx, smx, q.ds);
 }
@@ -1266,7 +1392,7 @@ void batch_block_counts(const Plan *p, int *nb) {
   nb[BATCH_PREP] = grid_for((long long)p->dim * N, kFlatPerBlock);
   for (int a = 0; a < 3; ++a) nb[BATCH_TRANSFER + a] = a < p->dim ? grid_for(p->nface_total[a], 256) : 0;
   nb[BATCH_DIVERGENCE] = g.nblk;
-  nb[BATCH_RESIDUAL] = (g.nblk + kResidualChunk - 1) / kResidualChunk;
+  nb[BATCH_RESIDUAL] = (pair_blocks(g) + kResidualChunk - 1) / kResidualChunk;
   nb[BATCH_GAUGE_SUM] = p->singular ? grid_for(nc, kFlatPerBlock) : 0;
   nb[BATCH_FINALIZE] = p->singular ? grid_for(nc, kFlatPerBlock) : 0;   // else split by the last pass
   nb[BATCH_GRADIENT] = grid_for(N, 256);
@@ -1286,6 +1412,7 @@ static BlockGrid block_grid(const Plan *p) {
 void batch_problem_fill(const Plan *p, const pc_project_args &a, BatchProblem &q) {
   memset(&q, 0, sizeof(q));
   q.g = grid_dev(p);
+  q.pair_blocks = pair_blocks(q.g);
   q.dim = p->dim; q.vdtype = p->vdtype; q.N = (int)p->N; q.ncells = (int)p->ncells; q.K = p->K; q.Kg = p->Kg;
   q.singular = p->singular;
   q.gmode = p->singular ? (p->gauge == 1 ? 2 : 1) : 0;
@@ -1397,7 +1524,20 @@ static void launch_residual(bool singular, bool write_r, bool norm, cudaStream_t
   // four rows per thread, the grid's own tiling: on the 256x128x128 box it took 0.194 ms for
   // three residuals against 0.290 ms with two rows per thread (the channel is unchanged)
   const GridDev g = g0;
-  const int grid = (g.nblk + (rs.chunk > 1 ? rs.chunk : 1) - 1) / (rs.chunk > 1 ? rs.chunk : 1);
+  const int per = rs.chunk > 1 ? rs.chunk : 1;
+  if constexpr (std::is_same<PV, float2>::value) {
+    // cell grids without L2 norms: two cells per thread (16-byte source: an FP64 one is the caller's)
+    const bool cells = g.lo_kind[0] < 2 && g.hi_kind[0] < 2 && g.lo_kind[g.dim - 1] < 2 && g.hi_kind[g.dim - 1] < 2 &&
+                       (g.dim == 2 || (g.lo_kind[1] < 2 && g.hi_kind[1] < 2));
+    if (write_r && !norm && cells && g.n[g.dim - 1] % 2 == 0 && ((uintptr_t)s & 15) == 0) {
+      const int nblk = pair_blocks(g), grid = (nblk + per - 1) / per;
+      auto k = g.dim == 2 ? (singular ? residual_pair_kernel<2, true, SV> : residual_pair_kernel<2, false, SV>)
+                          : (singular ? residual_pair_kernel<3, true, SV> : residual_pair_kernel<3, false, SV>);
+      launch_pdl(k, grid, 256, 0, st, g, s, p, r, ds, rs, nblk);
+      return;
+    }
+  }
+  const int grid = (g.nblk + per - 1) / per;
 #define PC_RES(S, W, N)                                                                                       \
   do {                                                                                                        \
     if (g.dim == 2)                                                                                           \
@@ -1584,6 +1724,22 @@ static void launch_gradient(Plan *p, cudaStream_t st, const double *dp, const vo
   }
 }
 
+// Face divergence of the transferred fluxes (pairs on mixed and FP32 plans, else FP64).
+static void launch_divergence(Plan *p, cudaStream_t st, const GridDev &gd, double inv_bdt, int sums) {
+  const double inc = 1.0 / (double)p->ncells;
+  if (p->precision != PC_PREC_FP64) {
+    const float2 *U[3] = {reinterpret_cast<const float2 *>(p->U64[0]), reinterpret_cast<const float2 *>(p->U64[1]),
+                          reinterpret_cast<const float2 *>(p->U64[2])};
+    auto k = p->dim == 2 ? divergence_kernel<2, float2> : divergence_kernel<3, float2>;
+    launch_pdl(k, gd.nblk, 256, 0, st, gd, U[0], U[1], U[2], inv_bdt, nullptr, reinterpret_cast<float2 *>(p->s64),
+               reinterpret_cast<float *>(p->work64), p->dstats, p->partials, p->counters, sums, inc);
+  } else {
+    auto k = p->dim == 2 ? divergence_kernel<2, double> : divergence_kernel<3, double>;
+    launch_pdl(k, gd.nblk, 256, 0, st, gd, p->U64[0], p->U64[1], p->U64[2], inv_bdt, p->s64, nullptr, nullptr, p->dstats,
+               p->partials, p->counters, sums, inc);
+  }
+}
+
 // Source of the direct-divergence mode into the same buffers as the face divergence.
 static void launch_direct_div(Plan *p, cudaStream_t st, double inv_bdt, int want_sums) {
   const bool mixed = p->precision != PC_PREC_FP64;
@@ -1683,9 +1839,10 @@ static pc_status project_impl(Plan *p, double dt, const void *u_star, const void
     const int G = grid_for(rows, T);
     if (mixed) {
       const PairSrc src{p->u2 + (long long)a * N};
-      if (p->K == 12) launch_pdl(transfer_mixed_kernel<12, PairSrc>, G, T, 0, st, (int)rows, p->K, p->fcol[a], p->fw2[a], src, p->U64[a]);
-      else if (p->K == 27) launch_pdl(transfer_mixed_kernel<27, PairSrc>, G, T, 0, st, (int)rows, p->K, p->fcol[a], p->fw2[a], src, p->U64[a]);
-      else launch_pdl(transfer_mixed_kernel<0, PairSrc>, G, T, 0, st, (int)rows, p->K, p->fcol[a], p->fw2[a], src, p->U64[a]);
+      float2 *U2 = reinterpret_cast<float2 *>(p->U64[a]);
+      if (p->K == 12) launch_pdl(transfer_mixed_kernel<12, PairSrc>, G, T, 0, st, (int)rows, p->K, p->fcol[a], p->fw2[a], src, U2);
+      else if (p->K == 27) launch_pdl(transfer_mixed_kernel<27, PairSrc>, G, T, 0, st, (int)rows, p->K, p->fcol[a], p->fw2[a], src, U2);
+      else launch_pdl(transfer_mixed_kernel<0, PairSrc>, G, T, 0, st, (int)rows, p->K, p->fcol[a], p->fw2[a], src, U2);
     } else {
       launch_pdl(transfer64_kernel, G, T, 0, st, (int)rows, p->K, p->fcol[a], p->fw64[a],
                  p->ut64 + (long long)a * N, p->U64[a]);
@@ -1695,13 +1852,8 @@ static pc_status project_impl(Plan *p, double dt, const void *u_star, const void
   GridDev g = grid_dev(p);
   if (p->divmode == PC_DIV_FACES) {
     prof_mark(p, st, 1);
-    auto divk = (d == 2) ? divergence_kernel<2> : divergence_kernel<3>;
     const int sums = stats ? 2 : (p->singular ? 1 : 0);
-    const GridDev gd = sums ? g : with_rows_per_thread(g, kSingleRows);
-    launch_pdl(divk, gd.nblk, 256, 0, st, gd, p->U64[0], p->U64[1], p->U64[2], 1.0 / (p->beta * dt),
-               mixed ? nullptr : p->s64, mixed ? reinterpret_cast<float2 *>(p->s64) : nullptr,
-               mixed ? reinterpret_cast<float *>(p->work64) : nullptr, p->dstats, p->partials, p->counters,
-               sums, 1.0 / (double)nc);
+    launch_divergence(p, st, sums ? g : with_rows_per_thread(g, kSingleRows), 1.0 / (p->beta * dt), sums);
     count_launch(p);
     prof_mark(p, st, 2);
   }
@@ -1751,8 +1903,15 @@ static pc_status project_impl(Plan *p, double dt, const void *u_star, const void
   count_launch(p);
   prof_mark(p, st, 6);
   if (stats && p->divmode == PC_DIV_FACES) {   // no face fluxes in the direct mode
-    auto chk = (d == 2) ? div_check_kernel<2> : div_check_kernel<3>;
-    launch_pdl(chk, g.nblk, 256, 0, st, g, p->U64[0], p->U64[1], p->U64[2], dp, p->beta * dt, p->dstats);
+    if (mixed) {
+      auto chk = (d == 2) ? div_check_kernel<2, float2> : div_check_kernel<3, float2>;
+      launch_pdl(chk, g.nblk, 256, 0, st, g, reinterpret_cast<const float2 *>(p->U64[0]),
+                 reinterpret_cast<const float2 *>(p->U64[1]), reinterpret_cast<const float2 *>(p->U64[2]), dp, p->beta * dt,
+                 p->dstats);
+    } else {
+      auto chk = (d == 2) ? div_check_kernel<2, double> : div_check_kernel<3, double>;
+      launch_pdl(chk, g.nblk, 256, 0, st, g, p->U64[0], p->U64[1], p->U64[2], dp, p->beta * dt, p->dstats);
+    }
     count_launch(p);
     prof_mark(p, st, 7);
   }
@@ -2064,14 +2223,15 @@ static pc_status ib_pass(Plan *p, bool first, double dt, const VT *du, double *d
     const int G = grid_for(nl, T);
     if (mixed) {
       const PairSrc src{p->u2 + (long long)a * N};
+      float2 *U2 = reinterpret_cast<float2 *>(p->U64[a]);
       if (first) {
-        if (p->K == 12) launch_pdl(transfer_mixed_kernel<12, PairSrc>, G, T, 0, st, (int)rows, p->K, p->fcol[a], p->fw2[a], src, p->U64[a]);
-        else if (p->K == 27) launch_pdl(transfer_mixed_kernel<27, PairSrc>, G, T, 0, st, (int)rows, p->K, p->fcol[a], p->fw2[a], src, p->U64[a]);
-        else launch_pdl(transfer_mixed_kernel<0, PairSrc>, G, T, 0, st, (int)rows, p->K, p->fcol[a], p->fw2[a], src, p->U64[a]);
+        if (p->K == 12) launch_pdl(transfer_mixed_kernel<12, PairSrc>, G, T, 0, st, (int)rows, p->K, p->fcol[a], p->fw2[a], src, U2);
+        else if (p->K == 27) launch_pdl(transfer_mixed_kernel<27, PairSrc>, G, T, 0, st, (int)rows, p->K, p->fcol[a], p->fw2[a], src, U2);
+        else launch_pdl(transfer_mixed_kernel<0, PairSrc>, G, T, 0, st, (int)rows, p->K, p->fcol[a], p->fw2[a], src, U2);
       } else {
-        if (p->K == 12) launch_pdl(ib_transfer_mixed_kernel<12>, G, T, 0, st, (int)nl, p->ib_face[a], (int)rows, p->K, p->fcol[a], p->fw2[a], src, p->U64[a]);
-        else if (p->K == 27) launch_pdl(ib_transfer_mixed_kernel<27>, G, T, 0, st, (int)nl, p->ib_face[a], (int)rows, p->K, p->fcol[a], p->fw2[a], src, p->U64[a]);
-        else launch_pdl(ib_transfer_mixed_kernel<0>, G, T, 0, st, (int)nl, p->ib_face[a], (int)rows, p->K, p->fcol[a], p->fw2[a], src, p->U64[a]);
+        if (p->K == 12) launch_pdl(ib_transfer_mixed_kernel<12>, G, T, 0, st, (int)nl, p->ib_face[a], (int)rows, p->K, p->fcol[a], p->fw2[a], src, U2);
+        else if (p->K == 27) launch_pdl(ib_transfer_mixed_kernel<27>, G, T, 0, st, (int)nl, p->ib_face[a], (int)rows, p->K, p->fcol[a], p->fw2[a], src, U2);
+        else launch_pdl(ib_transfer_mixed_kernel<0>, G, T, 0, st, (int)nl, p->ib_face[a], (int)rows, p->K, p->fcol[a], p->fw2[a], src, U2);
       }
     } else {
       if (first) launch_pdl(transfer64_kernel, G, T, 0, st, (int)rows, p->K, p->fcol[a], p->fw64[a], p->ut64 + (long long)a * N, p->U64[a]);
@@ -2082,12 +2242,7 @@ static pc_status ib_pass(Plan *p, bool first, double dt, const VT *du, double *d
   if (p->divmode == PC_DIV_FACES) {
     prof_mark(p, st, 1);
     GridDev g = grid_dev(p);
-    auto divk = (d == 2) ? divergence_kernel<2> : divergence_kernel<3>;
-    const GridDev gd = p->singular ? g : with_rows_per_thread(g, kSingleRows);
-    launch_pdl(divk, gd.nblk, 256, 0, st, gd, p->U64[0], p->U64[1], p->U64[2], 1.0 / (p->beta * dt),
-               mixed ? nullptr : p->s64, mixed ? reinterpret_cast<float2 *>(p->s64) : nullptr,
-               mixed ? reinterpret_cast<float *>(p->work64) : nullptr, p->dstats, p->partials, p->counters,
-               p->singular ? 1 : 0, 1.0 / (double)nc);
+    launch_divergence(p, st, p->singular ? g : with_rows_per_thread(g, kSingleRows), 1.0 / (p->beta * dt), p->singular ? 1 : 0);
     count_launch(p);
     prof_mark(p, st, 2);
   }

@@ -82,18 +82,6 @@ __device__ __forceinline__ void store_pairs(float2 *p, const Four &v) {
   *reinterpret_cast<float4 *>(p) = u;
   *reinterpret_cast<float4 *>(p + 2) = w;
 }
-__device__ __forceinline__ F2 f2_neg(F2 a) { return F2{a.v ^ 0x8000000080000000ULL}; }
-__device__ __forceinline__ DF2 df2_neg(DF2 a) { return DF2{f2_neg(a.hi), f2_neg(a.lo)}; }
-// The ghost of an edge value: itself (Neumann) or its negative (Dirichlet).
-__device__ __forceinline__ DF2 ghost(int kind, DF2 v) { return kind ? df2_neg(v) : v; }
-// (last of a, first of b): the pair between two neighbouring pairs.
-__device__ __forceinline__ F2 f2_mid(F2 a, F2 b) { return F2{(a.v >> 32) | (b.v << 32)}; }
-__device__ __forceinline__ DF2 df2_mid(DF2 a, DF2 b) { return DF2{f2_mid(a.hi, b.hi), f2_mid(a.lo, b.lo)}; }
-__device__ __forceinline__ float max_abs(float m, F2 v) {
-  float x, y;
-  f2_unpack(v, x, y);
-  return fmaxf(m, fmaxf(fabsf(x), fabsf(y)));
-}
 // pair_add (loop_pass.cuh) on two pairs.
 __device__ __forceinline__ DF2 pair_add2(DF2 old, F2 x) {
   const F2 s = f2_add(old.hi, x), z = f2_sub(s, old.hi);
