@@ -461,6 +461,9 @@ static void tables_of(const AxisInfo &ax, int &first, int &end) {
 // Largest grid of the cooperative solve: what the SMs' shared memory holds (1024^2: 135 us against
 // 258 by launches); the fit itself is checked for each plan.
 constexpr long long kResidentCells = 1LL << 20;
+// Grids that run as one cluster of 16 CTAs: the hardware barrier saves 1 us of each of about ten
+// barriers, at most two thousand cells per SM cost little of it again.
+constexpr long long kClusterCells = 1LL << 15;
 
 pc_status solve_resident(Plan *p, const double *s64, const float2 *s2, double *pout, int sweeps, bool adaptive,
                          float tol, const GridDev &g, cudaStream_t st, bool &taken) {
@@ -472,12 +475,14 @@ pc_status solve_resident(Plan *p, const double *s64, const float2 *s2, double *p
   }
   const void *rs = s2 ? (const void *)s2 : (const void *)s64;
   if (!aligned16(rs) || !aligned16(pout)) return PC_OK;
-  static const int sms = [] {
+  static const int all_sms = [] {
     int dev = 0, n = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
     return n;
   }();
+  const bool cluster = p->ncells <= kClusterCells && resident_cluster_size() > 0;
+  const int sms = cluster ? resident_cluster_size() : all_sms;
   const int np = 2 * p->dim - 1, last = p->dim - 1;
   ResidentArgs R;
   memset(&R, 0, sizeof(R));
@@ -522,6 +527,7 @@ pc_status solve_resident(Plan *p, const double *s64, const float2 *s2, double *p
     fits = smem <= (size_t)kResidentSmem;
   }
   if (!fits) return PC_OK;
+  R.cluster = cluster;
   for (int k = 0; k < np; ++k) {
     PassArgs<float> &A = R.pass[k];
     const AxisInfo &ax = p->ax[specs[k].axis];

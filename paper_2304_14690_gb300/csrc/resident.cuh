@@ -19,6 +19,7 @@ struct ResidentArgs {
   int tables_at;             // slots of shared memory before the tables
   int sweeps, adaptive, singular;
   int grid;                  // CTAs
+  int cluster;               // the grid is one cluster (small grids), else a cooperative launch
   int row_tiles;             // row tiles per CTA (consecutive)
   int own_at;                // slots of shared memory before the own rows' planes
   float tol;
@@ -26,5 +27,7 @@ struct ResidentArgs {
 
 pc_status launch_resident(const ResidentArgs &R, int dim, bool pairs, size_t smem, cudaStream_t st);
 pc_status prepare_resident();
+// CTAs of the largest cluster the kernel runs as (16, else 8; 0: none).
+int resident_cluster_size();
 
 }  // namespace pc
