@@ -242,8 +242,11 @@ static long long fill_loop(const Plan *p, const PassSpec &ps, PassArgs<Real> &A,
   return fill_tiles<Real>(p, A, L);
 }
 
+// Largest grid of the cooperative solve: what the SMs' shared memory holds (1024^2: 135 us against
+// 258 by launches); the fit itself is checked for each plan.
+constexpr long long kResidentCells = 1LL << 20;
 // Slots of a looped pass's tile: 2048 in FP32 (35 KB: six CTAs of 256 threads per SM) and 1024 in
-// FP64 in a launch of its own, up to 4096 on the resident CTAs.
+// FP64 in a launch of its own (4096: 64 2D problems 868 us against 823), up to 4096 on the resident CTAs.
 constexpr int kLoopSlots = 2048;
 
 static bool aligned16(const void *q) { return ((uintptr_t)q & 15) == 0; }
@@ -269,13 +272,18 @@ pc_status build_pass(const Plan *p, const PassSpec &ps, PassArgs<Real> &A, long 
   int E = fp32 ? ax.slots32 : ax.slots64;
   const bool deflt = fp32 ? E <= 1 : ax.loop64;
   const bool quad = quad_io(p, ps, fp32);
-  const bool lean = fp32 && deflt && pass_family(ax.kind) <= 2 && lean::length_ok(M) && quad;
+  bool all = true;   // an axis without a looped pass (odd M, vertex kinds): none on the others either
+  for (int a = 0; a < p->dim; ++a) all = all && p->ax[a].loop_nst > 0;
+  // variant 0 on grids beyond the cooperative solve (192^3: 871 us against 982 with looped passes);
+  // below, where many problems share a launch, one kernel for all their lengths and families is the
+  // better one (64 2D problems 845 us with up to six lean kernels side by side, 823 looped; 12
+  // requests 1572 and 1459). The bits are the same.
+  const bool lean = fp32 && deflt && pass_family(ax.kind) <= 2 && lean::length_ok(M) && quad &&
+                    (E == 1 || !all || p->ncells > kResidentCells);
   const int lv = E == 1 ? 1 : 0;
   // unrefined FP32 plans return the transforms' own rounding (1e-7): their bits stay those of the
   // general pass at the lengths without a compile-time one
   const bool unrefined = fp32 && p->precision == PC_PREC_FP32;
-  bool all = true;   // an axis without a looped pass (odd M, vertex kinds): the general passes on all
-  for (int a = 0; a < p->dim; ++a) all = all && p->ax[a].loop_nst > 0;
   if (deflt && !lean && quad && all && !unrefined) {
     // lines per tile: as many as the slots allow; a problem alone takes fewer where the GPU would
     // not be full (the lines do not depend on it)
@@ -458,9 +466,6 @@ static void tables_of(const AxisInfo &ax, int &first, int &end) {
   end = fam == 0 ? tw_quarter(M) : fam == 1 ? tw_dct4pre(M) : tw_total(M);
 }
 
-// Largest grid of the cooperative solve: what the SMs' shared memory holds (1024^2: 135 us against
-// 258 by launches); the fit itself is checked for each plan.
-constexpr long long kResidentCells = 1LL << 20;
 // Grids that run as one cluster of 16 CTAs: the hardware barrier saves 1 us of each of about ten
 // barriers, at most two thousand cells per SM cost little of it again.
 constexpr long long kClusterCells = 1LL << 15;
