@@ -467,31 +467,39 @@ __device__ __forceinline__ double trap_weight(const TrapWeights &w, long long c)
   return wt;
 }
 
-// Sum (weighted, see TrapWeights) and sum of squares of a cell array (the source of
-// pc_solve_poisson), and its mean.
+// Sum (weighted, see TrapWeights) of a cell array (the source of pc_solve_poisson) and its mean;
+// SQUARES: also the sum of squares (statistics). Mixed plans, whose refinement reads the mean on
+// every call, sum in double-float arithmetic (both sums in FP64 took 59 us on a 192^3 grid, on the
+// FP64 pipe); the others need the sums for statistics alone and take FP64.
+template <bool MIXED, bool SQUARES>
 __device__ __forceinline__ void sum_kernel_body(unsigned b, unsigned nblk, long long count, const double *x,
                                                 DevStats *stats, double *partials, unsigned int *counter,
                                                 const TrapWeights &w) {
+  DF d1{0.0f, 0.0f};
   double v1 = 0.0, v2 = 0.0;
 #pragma unroll
   for (int k = 0; k < kFlatPerThread; ++k) {
     const long long c = (long long)b * kFlatPerBlock + k * kFlatThreads + threadIdx.x;
     if (c < count) {
       const double v = x[c];
-      v1 += w.dim ? trap_weight(w, c) * v : v;
-      v2 = fma(v, v, v2);
+      const double wv = w.dim ? trap_weight(w, c) * v : v;   // a power of two: exact
+      if (MIXED) d1 = df_add(d1, df_of(wv));
+      else v1 += wv;
+      if (SQUARES) v2 = fma(v, v, v2);
     }
   }
   const VBlock vb{b, 0u, 0u, nblk, 1u, 1u};
+  if (MIXED) v1 = f2d_bits(d1.hi) + f2d_bits(d1.lo);
   if (grid_sum(v1, partials, counter, &stats->sum_s, vb))
     stats->mean_s = stats->sum_s / (w.dim ? w.total : (double)count);
-  grid_sum(v2, partials + nblk, counter + 1, &stats->sum_s2, vb);
+  if (SQUARES) grid_sum(v2, partials + nblk, counter + 1, &stats->sum_s2, vb);
 }
 
+template <bool MIXED, bool SQUARES>
 __global__ void sum_kernel(long long count, const double *x, DevStats *stats, double *partials,
                            unsigned int *counter, TrapWeights w) {
   pdl_enter();
-  sum_kernel_body(blockIdx.x, gridDim.x, count, x, stats, partials, counter, w);
+  sum_kernel_body<MIXED, SQUARES>(blockIdx.x, gridDim.x, count, x, stats, partials, counter, w);
 }
 
 // ----------------------------------------------------------------------------- residual
@@ -1565,6 +1573,15 @@ static void launch_residual(bool singular, bool write_r, bool norm, cudaStream_t
 // grid: no constant part in the DCT-I expansion), 2 zero first point. Problems with a zero mode
 // take the plan's gauge: the refinement cannot correct the constant that FP32 rounding leaves
 // (L_h of a constant is zero).
+// Whether a solve reads the mean of its source: the refinement's residual on zero-mode problems. The
+// transforms themselves drop the zero mode.
+static bool needs_mean(const Plan *p) { return p->singular && p->precision == PC_PREC_MIXED && p->refine_iters > 0; }
+
+static auto sum_kernel_of(const Plan *p, bool squares) {
+  if (p->precision == PC_PREC_MIXED) return squares ? sum_kernel<true, true> : sum_kernel<true, false>;
+  return squares ? sum_kernel<false, true> : sum_kernel<false, false>;
+}
+
 static int gauge_mode(const Plan *p) {
   if (!p->singular) return 0;
   return p->gauge == 1 ? 2 : 1;
@@ -1780,8 +1797,8 @@ static pc_status vertex_pass_solve(Plan *p, cudaStream_t st, double inv_bdt, dou
   count_launch(p);
   // the source sums: the (weighted) mean the residual removes on zero-mode problems, and the
   // statistics
-  if (want_stats || p->singular) {
-    launch_pdl(sum_kernel, grid_for(nc, kFlatPerBlock), kFlatThreads, 0, st, nc, (const double *)p->s64, p->dstats,
+  if (want_stats || needs_mean(p)) {
+    launch_pdl(sum_kernel_of(p, want_stats), grid_for(nc, kFlatPerBlock), kFlatThreads, 0, st, nc, (const double *)p->s64, p->dstats,
                p->partials, p->counters, trap_weights(p));
     count_launch(p);
   }
@@ -1833,7 +1850,7 @@ static pc_status project_impl(Plan *p, double dt, const void *u_star, const void
   if (p->vertex) {
     PC_TRY(vertex_pass_solve(p, st, 1.0 / (p->beta * dt), dp, stats != nullptr));
   } else if (p->divmode == PC_DIV_WLS_DIRECT) {
-    launch_direct_div(p, st, 1.0 / (p->beta * dt), stats ? 2 : (p->singular ? 1 : 0));
+    launch_direct_div(p, st, 1.0 / (p->beta * dt), stats ? 2 : (needs_mean(p) ? 1 : 0));
     count_launch(p);
     prof_mark(p, st, 2);
   }
@@ -1855,7 +1872,7 @@ static pc_status project_impl(Plan *p, double dt, const void *u_star, const void
   GridDev g = grid_dev(p);
   if (p->divmode == PC_DIV_FACES) {
     prof_mark(p, st, 1);
-    const int sums = stats ? 2 : (p->singular ? 1 : 0);
+    const int sums = stats ? 2 : (needs_mean(p) ? 1 : 0);
     launch_divergence(p, st, sums ? g : with_rows_per_thread(g, kSingleRows), 1.0 / (p->beta * dt), sums);
     count_launch(p);
     prof_mark(p, st, 2);
@@ -1930,13 +1947,9 @@ static pc_status project_impl(Plan *p, double dt, const void *u_star, const void
   return PC_OK;
 }
 
-// Grid-level solve of device arrays with a caller-built plan description (no staging, no
-// statistics): source sums, transform solve, gauge. Used by the allocation-free entry point.
+// Grid-level solve of device arrays with a caller-built plan description (FP64; no staging, no
+// statistics): transform solve, gauge. Used by the allocation-free entry point.
 pc_status solve_grid_device(Plan *p, const double *s, double *pout, cudaStream_t st) {
-  const long long nc = p->ncells;
-  launch_pdl(sum_kernel, grid_for(nc, kFlatPerBlock), kFlatThreads, 0, st, nc, s, p->dstats, p->partials, p->counters,
-             TrapWeights{});
-  count_launch(p);
   PC_CUDA_TRY(cudaGetLastError());
   return solve_grid(p, s, pout, false, st);
 }
@@ -1956,8 +1969,8 @@ static pc_status vertex_solve(Plan *p, const double *s, double *p_out, pc_stats 
   if (hp) dp = p->stage_p;
   prof_begin(p, st);
   PC_CUDA_TRY(cudaMemsetAsync(p->dstats, 0, sizeof(DevStats), st));
-  if (p->singular || stats) {   // the sums: the mean of a zero-mode problem, and the statistics
-    launch_pdl(sum_kernel, grid_for(nc, kFlatPerBlock), kFlatThreads, 0, st, nc, ds, p->dstats, p->partials,
+  if (needs_mean(p) || stats) {
+    launch_pdl(sum_kernel_of(p, stats != nullptr), grid_for(nc, kFlatPerBlock), kFlatThreads, 0, st, nc, ds, p->dstats, p->partials,
                p->counters, trap_weights(p));
     count_launch(p);
   }
@@ -1980,8 +1993,8 @@ static pc_status solve_impl(Plan *p, const double *s, double *p_out, pc_stats *s
   if (hp) dp = p->stage_p;
   prof_begin(p, st);
   PC_CUDA_TRY(cudaMemsetAsync(p->dstats, 0, sizeof(DevStats), st));
-  if (p->singular || stats) {   // the sums: the mean of a zero-mode problem, and the statistics
-    launch_pdl(sum_kernel, grid_for(nc, kFlatPerBlock), kFlatThreads, 0, st, nc, ds, p->dstats, p->partials, p->counters,
+  if (needs_mean(p) || stats) {
+    launch_pdl(sum_kernel_of(p, stats != nullptr), grid_for(nc, kFlatPerBlock), kFlatThreads, 0, st, nc, ds, p->dstats, p->partials, p->counters,
                TrapWeights{});
     count_launch(p);
   }
@@ -2215,7 +2228,7 @@ static pc_status ib_pass(Plan *p, bool first, double dt, const VT *du, double *d
   if (p->vertex) {                           // the whole source again, solve and restriction
     PC_TRY(vertex_pass_solve(p, st, 1.0 / (p->beta * dt), dp, false));
   } else if (p->divmode == PC_DIV_WLS_DIRECT) {   // the whole source again: no face lists in this mode
-    launch_direct_div(p, st, 1.0 / (p->beta * dt), p->singular ? 1 : 0);
+    launch_direct_div(p, st, 1.0 / (p->beta * dt), needs_mean(p) ? 1 : 0);
     count_launch(p);
     prof_mark(p, st, 2);
   }
@@ -2245,7 +2258,7 @@ static pc_status ib_pass(Plan *p, bool first, double dt, const VT *du, double *d
   if (p->divmode == PC_DIV_FACES) {
     prof_mark(p, st, 1);
     GridDev g = grid_dev(p);
-    launch_divergence(p, st, p->singular ? g : with_rows_per_thread(g, kSingleRows), 1.0 / (p->beta * dt), p->singular ? 1 : 0);
+    launch_divergence(p, st, needs_mean(p) ? g : with_rows_per_thread(g, kSingleRows), 1.0 / (p->beta * dt), needs_mean(p) ? 1 : 0);
     count_launch(p);
     prof_mark(p, st, 2);
   }
