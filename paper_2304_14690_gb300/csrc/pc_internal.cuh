@@ -386,6 +386,8 @@ GridDev grid_dev(const Plan *p);
 // s64. The iterate is left in p->p2 and, in FP64, in pout.
 pc_status solve_resident(Plan *p, const double *s64, const float2 *s2, double *pout, int sweeps, bool adaptive,
                          float tol, const GridDev &g, cudaStream_t st, bool &taken);
+// The plain FP64 solve of a small grid with its gauge (gauge_mode) as one launch (resident64.cu).
+pc_status solve_resident64(Plan *p, const double *s, double *pout, int gauge, cudaStream_t st, bool &taken);
 // Drops the plan's captured CUDA graphs and batch executables (after a schedule change).
 void plan_drop_graphs(Plan *p);
 // ----------------------------------------------------------------------------- batches

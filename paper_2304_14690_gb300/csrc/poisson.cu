@@ -283,8 +283,11 @@ pc_status build_pass(const Plan *p, const PassSpec &ps, PassArgs<Real> &A, long 
   const int lv = E == 1 ? 1 : 0;
   // unrefined FP32 plans return the transforms' own rounding (1e-7): their bits stay those of the
   // general pass at the lengths without a compile-time one
-  const bool unrefined = fp32 && p->precision == PC_PREC_FP32;
-  if (deflt && !lean && quad && all && !unrefined) {
+  const bool unrefined = fp32 && p->precision == PC_PREC_FP32 && !lean::length_ok(M);
+  // FP64 lines of 4096 values leave one CTA per SM its shared memory for (4096 x 128: 229 us against
+  // the general pass's 206; 2048 x 256: 160 against 238)
+  const bool too_long = !fp32 && M > 1024;
+  if (deflt && !lean && quad && all && !unrefined && !too_long) {
     // lines per tile: as many as the slots allow; a problem alone takes fewer where the GPU would
     // not be full (the lines do not depend on it)
     const int slots = fp32 ? kLoopSlots : kLoopSlots / 2;
@@ -423,6 +426,7 @@ pc_status prepare_kernels() {
   PC_TRY(prepare_lean(lim));
   PC_TRY(prepare_loop(lim));
   PC_TRY(prepare_resident());
+  PC_TRY(prepare_resident64());
   PC_TRY((prepare_axis_pass_spec<double, -1, false>(lim)));
   return PC_OK;
 }
@@ -466,34 +470,23 @@ static void tables_of(const AxisInfo &ax, int &first, int &end) {
   end = fam == 0 ? tw_quarter(M) : fam == 1 ? tw_dct4pre(M) : tw_total(M);
 }
 
-// Grids that run as one cluster of 16 CTAs: the hardware barrier saves 1 us of each of about ten
-// barriers, at most two thousand cells per SM cost little of it again.
-constexpr long long kClusterCells = 1LL << 15;
+// Grids that run as one cluster of 16 CTAs: the hardware barrier saves about 1 us at each of ten
+// barriers, the work of more cells per SM costs it again (2D: 128^2 43 us against 49 as a grid of
+// all SMs, 160 x 200 62 against 52; 3D: 20^3 80 against 84, 24^3 74 against 72).
+constexpr long long kClusterCells2D = 20000, kClusterCells3D = 8192;
+static bool cluster_grid(const Plan *p) {
+  return p->ncells <= (p->dim == 2 ? kClusterCells2D : kClusterCells3D) && resident_cluster_size() > 0;
+}
 
-pc_status solve_resident(Plan *p, const double *s64, const float2 *s2, double *pout, int sweeps, bool adaptive,
-                         float tol, const GridDev &g, cudaStream_t st, bool &taken) {
-  taken = false;
-  if (p->ncells > kResidentCells || sweeps > kMaxRefine) return PC_OK;
-  for (int a = 0; a < p->dim; ++a) {
-    if (p->ax[a].slots32 != 0 || p->ax[a].loop_nst == 0) return PC_OK;
-    if (p->precision == PC_PREC_FP32 && !lean::length_ok(p->ax[a].M)) return PC_OK;   // see build_pass
-  }
-  const void *rs = s2 ? (const void *)s2 : (const void *)s64;
-  if (!aligned16(rs) || !aligned16(pout)) return PC_OK;
-  static const int all_sms = [] {
-    int dev = 0, n = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    return n;
-  }();
-  const bool cluster = p->ncells <= kClusterCells && resident_cluster_size() > 0;
-  const int sms = cluster ? resident_cluster_size() : all_sms;
-  const int np = 2 * p->dim - 1, last = p->dim - 1;
-  ResidentArgs R;
-  memset(&R, 0, sizeof(R));
-  const std::vector<PassSpec> specs = solve_pass_specs(p, true, SRC_F32, rs, DST_PAIR_SET, p->p2);
-  // the tables behind the tiles: per axis the wrappers' factors its family reads, the stage twiddles
-  // and, on the dividing pass, the eigenvalues
+// Tiles, tables and own rows of a cooperative solve's passes: lines per tile as few as give every SM
+// at most one tile, and fewer again where the buffers would not leave room for the own rows
+// (own_bytes per cell). Behind the tiles: per axis the wrappers' factors its family reads, the stage
+// twiddles and, on the dividing pass, the eigenvalues.
+template <typename Real>
+static bool resident_layout(const Plan *p, const std::vector<PassSpec> &specs, PassArgs<Real> *pass, int sms, int cap0,
+                            int own_bytes, int &grid, int &row_tiles, int &tables_at, int &own_at, size_t &smem) {
+  constexpr int kSlot = 2 * (int)sizeof(Real);
+  const int np = (int)specs.size(), last = p->dim - 1;
   int slots = 0, at[3][3];
   for (int k = 0; k < p->dim; ++k) {
     const AxisInfo &ax = p->ax[specs[k].axis];
@@ -507,11 +500,8 @@ pc_status solve_resident(Plan *p, const double *s64, const float2 *s2, double *p
     if (specs[k].div) slots += (ax.n + 1) / 2;
   }
   slots = (slots + 1) & ~1;
-  // lines per tile: as few as give every SM at most one tile, and fewer again where
-  // the buffers would not leave room for the own rows
-  size_t smem = 0;
   bool fits = false;
-  for (int cap = 2 * kLoopSlots; cap >= kLoopSlots / 2 && !fits; cap /= 2) {
+  for (int cap = cap0; cap >= cap0 / 4 && !fits; cap /= 2) {
     long long most = 0;
     size_t tiles_smem = 0;
     for (int k = 0; k < np; ++k) {
@@ -519,22 +509,20 @@ pc_status solve_resident(Plan *p, const double *s64, const float2 *s2, double *p
       const long long lines = p->ncells / p->ax[specs[k].axis].n;
       int L = 1;
       while ((lines + L - 1) / L > sms && 2 * L * M <= cap) L *= 2;
-      const long long tiles = fill_loop<float>(p, specs[k], R.pass[k], L);
+      const long long tiles = fill_loop<Real>(p, specs[k], pass[k], L);
       most = tiles > most ? tiles : most;
-      const size_t b = loop::tile_smem<float>(M, L);
+      const size_t b = loop::tile_smem<Real>(M, L);
       tiles_smem = b > tiles_smem ? b : tiles_smem;
     }
-    R.grid = (int)(most < sms ? most : sms);
-    R.row_tiles = (R.pass[0].ntiles + R.grid - 1) / R.grid;
-    R.tables_at = (int)((tiles_smem + 15) / 16 * 2);
-    R.own_at = R.tables_at + slots;
-    smem = (size_t)R.own_at * sizeof(float2) + (size_t)R.row_tiles * R.pass[0].L * p->ax[last].n * 4 * sizeof(float);
+    grid = (int)(most < sms ? most : sms);
+    row_tiles = (pass[0].ntiles + grid - 1) / grid;
+    tables_at = (int)((tiles_smem + 15) / 16 * 16 / kSlot) + (kSlot == 8 ? 0 : 1);
+    own_at = tables_at + slots;
+    smem = (size_t)own_at * kSlot + (size_t)row_tiles * pass[0].L * p->ax[last].n * own_bytes;
     fits = smem <= (size_t)kResidentSmem;
   }
-  if (!fits) return PC_OK;
-  R.cluster = cluster;
   for (int k = 0; k < np; ++k) {
-    PassArgs<float> &A = R.pass[k];
+    PassArgs<Real> &A = pass[k];
     const AxisInfo &ax = p->ax[specs[k].axis];
     const int *t = at[specs[k].axis];
     tables_of(ax, A.tw_first, A.tw_last);
@@ -543,6 +531,37 @@ pc_status solve_resident(Plan *p, const double *s64, const float2 *s2, double *p
     A.st_count = loop_twiddles(ax);
     A.lam_at = t[2];
   }
+  return fits;
+}
+
+static int sm_count() {
+  static const int sms = [] {
+    int dev = 0, n = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    return n;
+  }();
+  return sms;
+}
+
+pc_status solve_resident(Plan *p, const double *s64, const float2 *s2, double *pout, int sweeps, bool adaptive,
+                         float tol, const GridDev &g, cudaStream_t st, bool &taken) {
+  taken = false;
+  if (p->ncells > kResidentCells || sweeps > kMaxRefine) return PC_OK;
+  for (int a = 0; a < p->dim; ++a) {
+    if (p->ax[a].slots32 != 0 || p->ax[a].loop_nst == 0) return PC_OK;
+    if (p->precision == PC_PREC_FP32 && !lean::length_ok(p->ax[a].M)) return PC_OK;   // see build_pass
+  }
+  const void *rs = s2 ? (const void *)s2 : (const void *)s64;
+  if (!aligned16(rs) || !aligned16(pout)) return PC_OK;
+  ResidentArgs R;
+  memset(&R, 0, sizeof(R));
+  R.cluster = cluster_grid(p);
+  size_t smem = 0;
+  if (!resident_layout<float>(p, solve_pass_specs(p, true, SRC_F32, rs, DST_PAIR_SET, p->p2), R.pass,
+                              R.cluster ? resident_cluster_size() : sm_count(), 2 * kLoopSlots, 16, R.grid, R.row_tiles,
+                              R.tables_at, R.own_at, smem))
+    return PC_OK;
   R.g = g;
   R.s = rs;
   R.p2 = p->p2;
@@ -554,6 +573,38 @@ pc_status solve_resident(Plan *p, const double *s64, const float2 *s2, double *p
   R.singular = p->singular;
   R.tol = tol;
   PC_TRY(launch_resident(R, p->dim, s2 != nullptr, smem, st));
+  count_launch(p);
+  taken = true;
+  return PC_OK;
+}
+
+// Largest grid of the FP64 solve in one launch (96^3 236 us against 275 by launches, 512^2 76 against
+// 80, 1024 x 96 41 against 57), and as one cluster (64^2 with a zero mode 31 against 33; beyond, the
+// FP64 pipes of 16 SMs are too few).
+constexpr long long kResident64Cells = 1LL << 20, kCluster64Cells = 4096;
+
+pc_status solve_resident64(Plan *p, const double *s, double *pout, int gauge, cudaStream_t st, bool &taken) {
+  taken = false;
+  if (p->ncells > kResident64Cells || !aligned16(s) || !aligned16(pout)) return PC_OK;
+  for (int a = 0; a < p->dim; ++a)
+    if (!p->ax[a].loop64 || p->ax[a].loop_nst == 0 || p->ax[a].M > 1024) return PC_OK;
+  Resident64Args R;
+  memset(&R, 0, sizeof(R));
+  R.cluster = p->ncells <= kCluster64Cells && resident_cluster_size() > 0;
+  size_t smem = 0;
+  if (!resident_layout<double>(p, solve_pass_specs(p, false, SRC_F64, s, DST_F64_SET, pout), R.pass,
+                               R.cluster ? resident_cluster_size() : sm_count(), kLoopSlots, 8, R.grid, R.row_tiles,
+                               R.tables_at, R.own_at, smem))
+    return PC_OK;
+  if (R.grid > 2 * (p->ncells / 256) + 64) return PC_OK;   // the partial sums' array (partial_slots)
+  R.s = s;
+  R.p = pout;
+  R.st = p->dstats;
+  R.partials = p->partials;
+  R.bar = p->dstats->bar;
+  R.gauge = gauge;
+  R.inv_cells = 1.0 / (double)p->ncells;
+  PC_TRY(launch_resident64(R, p->dim, smem, st));
   count_launch(p);
   taken = true;
   return PC_OK;

@@ -1592,8 +1592,12 @@ static pc_status solve_grid(Plan *p, const double *s64, double *pout, bool want_
   const long long nc = p->ncells;
   const int T = kFlatThreads;
   GridDev g = grid_dev(p);
+  int gmode = gauge_mode(p);
   if (p->precision == PC_PREC_FP64) {
-    PC_TRY(solve_fp64_grid(p, s64, pout, st));
+    bool resident = false;
+    PC_TRY(solve_resident64(p, s64, pout, gmode, st, resident));
+    if (resident) gmode = 0;   // applied
+    else PC_TRY(solve_fp64_grid(p, s64, pout, st));
     prof_mark(p, st, 3);
   } else {
     const int sweeps = (p->precision == PC_PREC_MIXED) ? p->refine_iters : 0;
@@ -1658,7 +1662,6 @@ static pc_status solve_grid(Plan *p, const double *s64, double *pout, bool want_
     prof_mark(p, st, 7);
   }
   // gauge, then the FP32 split of p for the mixed gradient
-  const int gmode = gauge_mode(p);
   if (gmode) {
     launch_pdl(gauge_sum_kernel, grid_for(nc, kFlatPerBlock), T, 0, st, nc, pout, p->dstats, p->partials, p->counters,
                gmode, trap_weights(p));

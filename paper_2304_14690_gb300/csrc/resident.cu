@@ -28,37 +28,6 @@ namespace pc {
 
 using loop::Quad;
 
-// Barrier of the whole grid (a cooperative launch: every CTA is resident). bar counts arrivals;
-// phase is the number of barriers passed. Bounded: after about two seconds it gives up, marks the
-// statistics and returns false (every CTA that waits does), and the caller leaves the kernel.
-__device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned &phase, DevStats *st) {
-  __shared__ int ok;
-  __syncthreads();
-  ++phase;
-  if (threadIdx.x == 0) {
-    const unsigned want = phase * gridDim.x;
-    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
-    unsigned seen = 0;
-    int good = 0;
-    for (int it = 0; it < (1 << 22); ++it) {
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
-      if (seen >= want) {
-        good = 1;
-        break;
-      }
-    }
-    if (!good) atomicOr(&st->flags, (unsigned)FLAG_TIMEOUT);
-    ok = good;
-  }
-  __syncthreads();
-  return ok != 0;
-}
-
-// Barrier of a grid that is one cluster: the hardware's (0.2 us against 1.2 for the grid barrier).
-__device__ __forceinline__ void cluster_barrier() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
 // Four consecutive values as two packed pairs: from global memory past L1 (other CTAs write it), or
 // from the planes of high and low parts in shared memory.
 struct Four { DF2 a, b; };

@@ -25,9 +25,57 @@ struct ResidentArgs {
   float tol;
 };
 
+// The plain FP64 solve of a small grid: its passes, the gauge and p in one launch (resident64.cu).
+struct Resident64Args {
+  PassArgs<double> pass[5];
+  const double *s;
+  double *p;
+  DevStats *st;
+  double *partials;          // one sum of p per CTA
+  unsigned *bar;
+  int grid, cluster, row_tiles, tables_at, own_at;
+  int gauge;                 // 0 none, 1 zero mean, 2 zero first cell
+  double inv_cells;
+};
+pc_status launch_resident64(const Resident64Args &R, int dim, size_t smem, cudaStream_t st);
+pc_status prepare_resident64();
+
 pc_status launch_resident(const ResidentArgs &R, int dim, bool pairs, size_t smem, cudaStream_t st);
 pc_status prepare_resident();
 // CTAs of the largest cluster the kernel runs as (16, else 8; 0: none).
 int resident_cluster_size();
+
+#ifdef __CUDACC__
+// Barrier of the whole grid (a cooperative launch: every CTA is resident). bar counts arrivals;
+// phase is the number of barriers passed. Bounded: after about two seconds it gives up, marks the
+// statistics and returns false (every CTA that waits does), and the caller leaves the kernel.
+__device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned &phase, DevStats *st) {
+  __shared__ int ok;
+  __syncthreads();
+  ++phase;
+  if (threadIdx.x == 0) {
+    const unsigned want = phase * gridDim.x;
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+    unsigned seen = 0;
+    int good = 0;
+    for (int it = 0; it < (1 << 22); ++it) {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
+      if (seen >= want) {
+        good = 1;
+        break;
+      }
+    }
+    if (!good) atomicOr(&st->flags, (unsigned)FLAG_TIMEOUT);
+    ok = good;
+  }
+  __syncthreads();
+  return ok != 0;
+}
+
+// Barrier of a grid that is one cluster: the hardware's (0.2 us against 1.2 for the grid barrier).
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+#endif
 
 }  // namespace pc

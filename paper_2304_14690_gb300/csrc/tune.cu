@@ -24,8 +24,12 @@ static bool valid_ctas(int c) { return c == 1 || c == 2 || c == 4 || c == 8; }
 
 // One solve of the plan's transform precision from s64 into the staging buffer.
 static pc_status run_solve(Plan *p, bool fp64, cudaStream_t st) {
-  if (fp64) return solve_fp64_grid(p, p->s64, p->stage_p, st);
-  bool taken = false;   // grids of the cooperative solve: one launch under the default schedule
+  bool taken = false;
+  if (fp64) {
+    PC_TRY(solve_resident64(p, p->s64, p->stage_p, 0, st, taken));
+    return taken ? PC_OK : solve_fp64_grid(p, p->s64, p->stage_p, st);
+  }
+  // grids of the cooperative solve: one launch under the default schedule
   PC_TRY(solve_resident(p, p->s64, nullptr, p->stage_p, 0, false, 0.0f, grid_dev(p), st, taken));
   if (taken) return PC_OK;
   return solve_fp32_grid(p, SRC_F64, p->s64, DST_F64_SET, p->stage_p, st);
