@@ -257,9 +257,8 @@ pc_status record_exec(Exec *e, cudaStream_t st, Plan *prof = nullptr) {
   if (prof) prof_begin(prof, st);
   for (const Group &g : e->groups) {
     const int n = (int)g.members.size();
-    batch_launch(BATCH_ZERO, 0, g.dP, nullptr, n, n, 0, st);
     batch_launch(BATCH_PREP, g.vdtype, g.dP, segs(g, BATCH_PREP), n, g.total[BATCH_PREP], 0, st);
-    launches += 2;
+    ++launches;
   }
   mark(0);
   for (const Group &g : e->groups)

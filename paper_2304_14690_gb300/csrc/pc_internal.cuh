@@ -393,7 +393,7 @@ void plan_drop_graphs(Plan *p);
 // ----------------------------------------------------------------------------- batches
 // Stages of the batched pipeline (one launch per stage for all problems of a batch).
 enum BatchStage {
-  BATCH_ZERO = 0, BATCH_PREP = 1, BATCH_TRANSFER = 2 /* +axis */, BATCH_DIVERGENCE = 5, BATCH_RESIDUAL = 6,
+  BATCH_PREP = 1, BATCH_TRANSFER = 2 /* +axis */, BATCH_DIVERGENCE = 5, BATCH_RESIDUAL = 6,
   BATCH_GAUGE_SUM = 7, BATCH_FINALIZE = 8, BATCH_GRADIENT = 9, BATCH_STAGES = 10
 };
 

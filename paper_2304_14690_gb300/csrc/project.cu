@@ -157,10 +157,19 @@ constexpr int kFlatThreads = 256;
 constexpr int kFlatPerThread = 4;
 constexpr int kFlatPerBlock = kFlatThreads * kFlatPerThread;
 
+// Without STATS the first block clears the call's device statistics (no memset node before the first
+// kernel: 1.5 us of a small projection); with them the host clears them first, since every block
+// merges its maximum.
+__device__ __forceinline__ void clear_stats(DevStats *st) {
+  unsigned *w = reinterpret_cast<unsigned *>(st);
+  for (int k = threadIdx.x; k < (int)(sizeof(DevStats) / 4); k += blockDim.x) w[k] = 0u;
+}
+
 template <typename VT, bool HAS_F, bool STATS, bool SPLIT>
 __device__ __forceinline__ void prep_kernel_body(unsigned b, long long count, const VT *__restrict__ u, const VT *__restrict__ f, double dt,
                             double *__restrict__ ut64, float2 *__restrict__ u2, DevStats *stats) {
   double m = 0.0;
+  if (!STATS && stats && b == 0) clear_stats(stats);
 #pragma unroll
   for (int k = 0; k < kFlatPerThread; ++k) {
     const long long i = (long long)b * kFlatPerBlock + k * kFlatThreads + threadIdx.x;
@@ -1049,8 +1058,9 @@ __global__ void ib_gather_kernel(int nib, int N, int dim, const int32_t *__restr
 template <typename VT, bool SPLIT>
 __global__ void ib_prep_kernel(int nib, int N, int dim, const int32_t *__restrict__ idx,
                                const VT *__restrict__ u, const VT *__restrict__ fc, VT *__restrict__ fo,
-                               double dt, double *__restrict__ ut64, float2 *__restrict__ u2) {
+                               double dt, double *__restrict__ ut64, float2 *__restrict__ u2, DevStats *clear) {
   pdl_enter();
+  if (clear && blockIdx.x == 0) clear_stats(clear);   // a later pass: its statistics start here
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= nib) return;
   const int i = __ldg(idx + j);
@@ -1258,12 +1268,6 @@ __device__ __forceinline__ VBlock flat_block(int local, int nblocks) {
   return VBlock{(unsigned)local, 0u, 0u, (unsigned)nblocks, 1u, 1u};
 }
 
-__global__ void batch_zero_stats(const BatchProblem *__restrict__ P) {
-  pdl_enter();
-  unsigned *w = reinterpret_cast<unsigned *>(P[blockIdx.x].ds);
-  for (int k = threadIdx.x; k < (int)(sizeof(DevStats) / 4); k += blockDim.x) w[k] = 0u;
-}
-
 template <typename VT>
 __global__ void batch_prep(const BatchProblem *__restrict__ P, const int *__restrict__ seg, int count) {
   pdl_enter();
@@ -1271,8 +1275,8 @@ __global__ void batch_prep(const BatchProblem *__restrict__ P, const int *__rest
   const BatchProblem &q = P[pi];
   const unsigned lb = blockIdx.x - seg[pi];
   const long long cnt = (long long)q.dim * q.N;
-  if (q.f) prep_kernel_body<VT, true, false, true>(lb, cnt, (const VT *)q.u, (const VT *)q.f, q.dt, nullptr, q.u2, nullptr);
-  else prep_kernel_body<VT, false, false, true>(lb, cnt, (const VT *)q.u, nullptr, q.dt, nullptr, q.u2, nullptr);
+  if (q.f) prep_kernel_body<VT, true, false, true>(lb, cnt, (const VT *)q.u, (const VT *)q.f, q.dt, nullptr, q.u2, q.ds);
+  else prep_kernel_body<VT, false, false, true>(lb, cnt, (const VT *)q.u, nullptr, q.dt, nullptr, q.u2, q.ds);
 }
 
 template <int KC>
@@ -1366,7 +1370,6 @@ void batch_launch(int stage, int variant, const BatchProblem *P, const int *seg,
   if (total_blocks <= 0) return;
   const int T = 256;
   switch (stage) {
-    case BATCH_ZERO: launch_pdl(batch_zero_stats, count, 64, 0, st, P); break;
     case BATCH_PREP:
       if (variant == PC_DTYPE_F64) launch_pdl(batch_prep<double>, total_blocks, T, 0, st, P, seg, count);
       else launch_pdl(batch_prep<float>, total_blocks, T, 0, st, P, seg, count);
@@ -1399,7 +1402,7 @@ void batch_launch(int stage, int variant, const BatchProblem *P, const int *seg,
 void batch_block_counts(const Plan *p, int *nb) {
   const long long N = p->N, nc = p->ncells;
   const GridDev g = grid_dev(p);
-  nb[BATCH_ZERO] = 1;
+  nb[0] = 0;
   nb[BATCH_PREP] = grid_for((long long)p->dim * N, kFlatPerBlock);
   for (int a = 0; a < 3; ++a) nb[BATCH_TRANSFER + a] = a < p->dim ? grid_for(p->nface_total[a], 256) : 0;
   nb[BATCH_DIVERGENCE] = g.nblk;
@@ -1838,7 +1841,7 @@ static pc_status project_impl(Plan *p, double dt, const void *u_star, const void
   if (f_out && hfo) dfo = p->stage_fo;
 
   prof_begin(p, st);
-  PC_CUDA_TRY(cudaMemsetAsync(p->dstats, 0, sizeof(DevStats), st));
+  if (stats) PC_CUDA_TRY(cudaMemsetAsync(p->dstats, 0, sizeof(DevStats), st));   // else by the prep kernel
   const int T = 256;
   const bool mixed = p->precision != PC_PREC_FP64;
   const long long cnt = (long long)d * N;
@@ -2217,14 +2220,13 @@ static pc_status ib_pass(Plan *p, bool first, double dt, const VT *du, double *d
   const int nib = (int)p->nib;
   VT *fo = static_cast<VT *>(p->ib_f[0]), *fc = static_cast<VT *>(p->ib_f[1]);
   prof_begin(p, st);
-  PC_CUDA_TRY(cudaMemsetAsync(p->dstats, 0, sizeof(DevStats), st));
-  if (first) {
+  if (first) {   // clears the statistics, as the IB nodes' prep does on later passes
     launch_prep<VT>(false, false, mixed, (long long)d * N, du, nullptr, dt, p->ut64, p->u2, p->dstats, st);
     count_launch(p);
   }
   if (nib) {
-    if (mixed) launch_pdl(ib_prep_kernel<VT, true>, grid_for(nib, T), T, 0, st, nib, (int)N, d, p->ib_idx, du, (const VT *)fc, fo, dt, p->ut64, p->u2);
-    else launch_pdl(ib_prep_kernel<VT, false>, grid_for(nib, T), T, 0, st, nib, (int)N, d, p->ib_idx, du, (const VT *)fc, fo, dt, p->ut64, p->u2);
+    if (mixed) launch_pdl(ib_prep_kernel<VT, true>, grid_for(nib, T), T, 0, st, nib, (int)N, d, p->ib_idx, du, (const VT *)fc, fo, dt, p->ut64, p->u2, first ? nullptr : p->dstats);
+    else launch_pdl(ib_prep_kernel<VT, false>, grid_for(nib, T), T, 0, st, nib, (int)N, d, p->ib_idx, du, (const VT *)fc, fo, dt, p->ut64, p->u2, first ? nullptr : p->dstats);
     count_launch(p);
   }
   prof_mark(p, st, 0);
