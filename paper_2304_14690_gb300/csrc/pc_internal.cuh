@@ -384,6 +384,7 @@ GridDev grid_dev(const Plan *p);
 // The refined FP32 solve as one cooperative kernel (resident.cu) where the plan and the arrays allow
 // it; taken says whether it was launched. s2 (nullable): the source as (hi, lo) pairs, else FP64 in
 // s64. The iterate is left in p->p2 and, in FP64, in pout.
+pc_status solve_fixed_sweeps(Plan *p, const double *s64, double *pout, int sweeps, cudaStream_t st);
 pc_status solve_resident(Plan *p, const double *s64, const float2 *s2, double *pout, int sweeps, bool adaptive,
                          float tol, const GridDev &g, cudaStream_t st, bool &taken);
 // The plain FP64 solve of a small grid with its gauge (gauge_mode) as one launch (resident64.cu).

@@ -1682,6 +1682,24 @@ static pc_status solve_grid(Plan *p, const double *s64, double *pout, bool want_
   return PC_OK;
 }
 
+// A solve of a mixed plan with a fixed number of sweeps and no gauge, whatever the source holds: what
+// the autotuner times.
+pc_status solve_fixed_sweeps(Plan *p, const double *s64, double *pout, int sweeps, cudaStream_t st) {
+  const GridDev g = grid_dev(p);
+  bool taken = false;
+  PC_TRY(solve_resident(p, s64, nullptr, pout, sweeps, false, 0.0f, g, st, taken));
+  if (taken) return PC_OK;
+  PC_TRY(solve_fp32_grid(p, SRC_F64_, s64, DST_PAIR_SET_, p->p2, st, sweeps == 0 ? pout : nullptr));
+  float *r32 = reinterpret_cast<float *>(p->work64);
+  for (int it = 0; it < sweeps; ++it) {
+    launch_residual(p->singular, true, false, st, g, s64, (const float2 *)p->p2, r32, p->dstats, &p->dstats->res2[it],
+                    p->partials, p->counters, RefineStep{it, 0, 0.0f, 1});
+    count_launch(p);
+    PC_TRY(solve_fp32_grid(p, SRC_F32_, r32, DST_PAIR_ADD_, p->p2, st, it == sweeps - 1 ? pout : nullptr));
+  }
+  return PC_OK;
+}
+
 static pc_status fill_stats(Plan *p, pc_stats *stats, cudaStream_t st) {
   DevStats ds;
   PC_CUDA_TRY(cudaMemcpyAsync(&ds, p->dstats, sizeof(DevStats), cudaMemcpyDeviceToHost, st));

@@ -22,6 +22,13 @@ static int &ctas_ref(Plan *p, int axis, bool fp64) {
 }
 static bool valid_ctas(int c) { return c == 1 || c == 2 || c == 4 || c == 8; }
 
+// Sweeps of the timed solve: a refined plan's first two, which is what the stopping rule mostly leaves.
+// Without them the 1024 x 512 channel's one-launch solve could lose to launches of variant 1, whose
+// transforms alone are about as fast; per projection these take 185 us against 129.
+static int tuned_sweeps(const Plan *p) {
+  return p->precision == PC_PREC_MIXED ? (p->refine_iters < 2 ? p->refine_iters : 2) : 0;
+}
+
 // One solve of the plan's transform precision from s64 into the staging buffer.
 static pc_status run_solve(Plan *p, bool fp64, cudaStream_t st) {
   bool taken = false;
@@ -29,6 +36,7 @@ static pc_status run_solve(Plan *p, bool fp64, cudaStream_t st) {
     PC_TRY(solve_resident64(p, p->s64, p->stage_p, 0, st, taken));
     return taken ? PC_OK : solve_fp64_grid(p, p->s64, p->stage_p, st);
   }
+  if (tuned_sweeps(p) > 0) return solve_fixed_sweeps(p, p->s64, p->stage_p, tuned_sweeps(p), st);
   // grids of the cooperative solve: one launch under the default schedule
   PC_TRY(solve_resident(p, p->s64, nullptr, p->stage_p, 0, false, 0.0f, grid_dev(p), st, taken));
   if (taken) return PC_OK;
@@ -62,7 +70,7 @@ static pc_status autotune(Plan *p, cudaStream_t st, double *best_out) {
   }
   pc_status status = PC_OK;
   float best = 0.0f;
-  const int reps = p->ncells > (1 << 22) ? 3 : (p->ncells > (1 << 18) ? 10 : 30);
+  const int reps = (p->ncells > (1 << 22) ? 3 : (p->ncells > (1 << 18) ? 12 : 30)) / (1 + tuned_sweeps(p));
   if (cudaMemsetAsync(p->s64, 0, p->ncells * sizeof(double), st) != cudaSuccess ||
       cudaMemsetAsync(p->dstats, 0, sizeof(DevStats), st) != cudaSuccess)
     status = fail(PC_ERR_CUDA, "cudaMemsetAsync failed");
