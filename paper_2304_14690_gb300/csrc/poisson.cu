@@ -296,7 +296,7 @@ pc_status build_pass(const Plan *p, const PassSpec &ps, PassArgs<Real> &A, long 
     if (batch_threads <= 0) {
       const long long lines = p->ncells / ax.n;
       while (L > 4 && lines / L < 2 * 152) L /= 2;
-      while (L > 1 && lines / L < 152) L /= 2;   // few long lines (1024 x 96 in FP64: 152 us at four, start 86)
+      while (L > 1 && lines / L < 152) L /= 2;   // few long lines (1024 x 96 in FP64: 152 us at four lines, 57 at one)
     }
     while (L > 1 && loop::tile_smem<Real>(M, L) > 160 * 1024) L /= 2;
     tiles = fill_loop<Real>(p, ps, A, L);

@@ -238,8 +238,13 @@ __global__ void transfer64_kernel(int rows, int K, const int32_t *__restrict__ c
 // The gathers' registers are bounded for the number of warps that keeps most bytes in flight: 32
 // (2D: eight CTAs of 256 threads per SM) and 48 registers (3D transfers: five; unbounded the
 // compiler takes 53 to 124), 32 and 40 for the gradients. 256x128x128 box: 1857 -> 1639 us.
-// The gathered node value as an FP32 (hi, lo) pair, here the pairs of u~ that prep wrote.
+// The gathered node value as an FP32 (hi, lo) pair, here the pairs of u~ that prep wrote. F64: the
+// plan's solve is not refined, so the last bit of the source's FP32 copy shows in the result (4.8e-8
+// of p over 24 problems), and the fluxes take the rounding to FP64 that they always had there. A
+// template argument: as a flag tested per row it cost 64 2D problems 15 of 832 us.
+template <bool F64>
 struct PairSrc {
+  static constexpr bool kF64 = F64;
   const float2 *p;
   __device__ __forceinline__ float2 operator()(int c) const { return __ldg(p + c); }
 };
@@ -268,6 +273,10 @@ __device__ __forceinline__ float2 transfer_mixed_row(int r, int rows, int Kr, co
   }
   // the flux stays a pair, renormalised without error (TwoSum): the divergence takes pairs
   float hi, lo;
+  if constexpr (Src::kF64) {
+    split_f64(df_value(s), hi, lo);
+    return make_float2(hi, lo);
+  }
   two_sum(s.hi, s.lo, hi, lo);
   return make_float2(hi, lo);
 }
@@ -1084,10 +1093,10 @@ __global__ void ib_transfer64_kernel(int nl, const int32_t *__restrict__ list, i
   const int r = __ldg(list + t);
   U[r] = transfer64_row(r, rows, K, col, w, u);
 }
-template <int KC>
+template <int KC, typename Src>
 __global__ void ib_transfer_mixed_kernel(int nl, const int32_t *__restrict__ list, int rows, int Kr,
                                          const int32_t *__restrict__ col, const float2 *__restrict__ w2,
-                                         PairSrc src, float2 *__restrict__ U) {
+                                         Src src, float2 *__restrict__ U) {
   pdl_enter();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= nl) return;
@@ -1279,13 +1288,13 @@ __global__ void batch_prep(const BatchProblem *__restrict__ P, const int *__rest
   else prep_kernel_body<VT, false, false, true>(lb, cnt, (const VT *)q.u, nullptr, q.dt, nullptr, q.u2, q.ds);
 }
 
-template <int KC>
+template <int KC, bool F64>
 __global__ void __launch_bounds__(256, KC == 12 ? 8 : KC == 27 ? 5 : 1) batch_transfer(const BatchProblem *__restrict__ P, const int *__restrict__ seg, int count, int a) {
   pdl_enter();
   const int pi = batch_problem_of(seg, count, blockIdx.x);
   const BatchProblem &q = P[pi];
   const VBlock vb = flat_block(blockIdx.x - seg[pi], seg[pi + 1] - seg[pi]);
-  transfer_mixed_kernel_body<KC>(vb, q.frows[a], q.K, q.fcol[a], q.fw2[a], PairSrc{q.u2 + (long long)a * q.N},
+  transfer_mixed_kernel_body<KC>(vb, q.frows[a], q.K, q.fcol[a], q.fw2[a], PairSrc<F64>{q.u2 + (long long)a * q.N},
                                  reinterpret_cast<float2 *>(q.U64[a]));
 }
 
@@ -1374,10 +1383,14 @@ void batch_launch(int stage, int variant, const BatchProblem *P, const int *seg,
       if (variant == PC_DTYPE_F64) launch_pdl(batch_prep<double>, total_blocks, T, 0, st, P, seg, count);
       else launch_pdl(batch_prep<float>, total_blocks, T, 0, st, P, seg, count);
       break;
-    case BATCH_TRANSFER:
-      if (variant == 12) launch_pdl(batch_transfer<12>, total_blocks, T, 0, st, P, seg, count, extra);
-      else if (variant == 27) launch_pdl(batch_transfer<27>, total_blocks, T, 0, st, P, seg, count, extra);
-      else launch_pdl(batch_transfer<0>, total_blocks, T, 0, st, P, seg, count, extra);
+    case BATCH_TRANSFER:   // variant: K, negative for unrefined plans
+      if (variant < 0) {   // the problems of a group share their sweeps: none
+        auto k = variant == -12 ? batch_transfer<12, true> : (variant == -27 ? batch_transfer<27, true> : batch_transfer<0, true>);
+        launch_pdl(k, total_blocks, T, 0, st, P, seg, count, extra);
+      } else {
+        auto k = variant == 12 ? batch_transfer<12, false> : (variant == 27 ? batch_transfer<27, false> : batch_transfer<0, false>);
+        launch_pdl(k, total_blocks, T, 0, st, P, seg, count, extra);
+      }
       break;
     case BATCH_DIVERGENCE:   // variant: the group's dimension
       if (variant == 3) launch_pdl(batch_divergence<3>, total_blocks, T, 0, st, P, seg, count);
@@ -1576,6 +1589,23 @@ static void launch_residual(bool singular, bool write_r, bool norm, cudaStream_t
 // grid: no constant part in the DCT-I expansion), 2 zero first point. Problems with a zero mode
 // take the plan's gauge: the refinement cannot correct the constant that FP32 rounding leaves
 // (L_h of a constant is zero).
+static bool unrefined(const Plan *p) { return p->precision == PC_PREC_FP32 || p->refine_iters == 0; }
+
+// Fluxes of axis a: every face row, or the nl listed ones that an IB node reaches (nl >= 0).
+template <bool F64>
+static void launch_transfer(const Plan *p, int a, long long nl, cudaStream_t st) {
+  using Src = PairSrc<F64>;
+  const Src src{p->u2 + (long long)a * p->N};
+  const int rows = (int)p->nface_total[a], T = 256, G = grid_for(nl < 0 ? rows : nl, T);
+  float2 *U = reinterpret_cast<float2 *>(p->U64[a]);
+  if (nl < 0) {
+    auto k = p->K == 12 ? transfer_mixed_kernel<12, Src> : (p->K == 27 ? transfer_mixed_kernel<27, Src> : transfer_mixed_kernel<0, Src>);
+    launch_pdl(k, G, T, 0, st, rows, p->K, p->fcol[a], p->fw2[a], src, U);
+  } else {
+    auto k = p->K == 12 ? ib_transfer_mixed_kernel<12, Src> : (p->K == 27 ? ib_transfer_mixed_kernel<27, Src> : ib_transfer_mixed_kernel<0, Src>);
+    launch_pdl(k, G, T, 0, st, (int)nl, p->ib_face[a], rows, p->K, p->fcol[a], p->fw2[a], src, U);
+  }
+}
 // Whether a solve reads the mean of its source: the refinement's residual on zero-mode problems. The
 // transforms themselves drop the zero mode.
 static bool needs_mean(const Plan *p) { return p->singular && p->precision == PC_PREC_MIXED && p->refine_iters > 0; }
@@ -1882,11 +1912,8 @@ static pc_status project_impl(Plan *p, double dt, const void *u_star, const void
     const long long rows = p->nface_total[a];
     const int G = grid_for(rows, T);
     if (mixed) {
-      const PairSrc src{p->u2 + (long long)a * N};
-      float2 *U2 = reinterpret_cast<float2 *>(p->U64[a]);
-      if (p->K == 12) launch_pdl(transfer_mixed_kernel<12, PairSrc>, G, T, 0, st, (int)rows, p->K, p->fcol[a], p->fw2[a], src, U2);
-      else if (p->K == 27) launch_pdl(transfer_mixed_kernel<27, PairSrc>, G, T, 0, st, (int)rows, p->K, p->fcol[a], p->fw2[a], src, U2);
-      else launch_pdl(transfer_mixed_kernel<0, PairSrc>, G, T, 0, st, (int)rows, p->K, p->fcol[a], p->fw2[a], src, U2);
+      if (unrefined(p)) launch_transfer<true>(p, a, -1, st);
+      else launch_transfer<false>(p, a, -1, st);
     } else {
       launch_pdl(transfer64_kernel, G, T, 0, st, (int)rows, p->K, p->fcol[a], p->fw64[a],
                  p->ut64 + (long long)a * N, p->U64[a]);
@@ -2261,17 +2288,8 @@ static pc_status ib_pass(Plan *p, bool first, double dt, const VT *du, double *d
     if (nl == 0) continue;
     const int G = grid_for(nl, T);
     if (mixed) {
-      const PairSrc src{p->u2 + (long long)a * N};
-      float2 *U2 = reinterpret_cast<float2 *>(p->U64[a]);
-      if (first) {
-        if (p->K == 12) launch_pdl(transfer_mixed_kernel<12, PairSrc>, G, T, 0, st, (int)rows, p->K, p->fcol[a], p->fw2[a], src, U2);
-        else if (p->K == 27) launch_pdl(transfer_mixed_kernel<27, PairSrc>, G, T, 0, st, (int)rows, p->K, p->fcol[a], p->fw2[a], src, U2);
-        else launch_pdl(transfer_mixed_kernel<0, PairSrc>, G, T, 0, st, (int)rows, p->K, p->fcol[a], p->fw2[a], src, U2);
-      } else {
-        if (p->K == 12) launch_pdl(ib_transfer_mixed_kernel<12>, G, T, 0, st, (int)nl, p->ib_face[a], (int)rows, p->K, p->fcol[a], p->fw2[a], src, U2);
-        else if (p->K == 27) launch_pdl(ib_transfer_mixed_kernel<27>, G, T, 0, st, (int)nl, p->ib_face[a], (int)rows, p->K, p->fcol[a], p->fw2[a], src, U2);
-        else launch_pdl(ib_transfer_mixed_kernel<0>, G, T, 0, st, (int)nl, p->ib_face[a], (int)rows, p->K, p->fcol[a], p->fw2[a], src, U2);
-      }
+      if (unrefined(p)) launch_transfer<true>(p, a, first ? -1 : nl, st);
+      else launch_transfer<false>(p, a, first ? -1 : nl, st);
     } else {
       if (first) launch_pdl(transfer64_kernel, G, T, 0, st, (int)rows, p->K, p->fcol[a], p->fw64[a], p->ut64 + (long long)a * N, p->U64[a]);
       else launch_pdl(ib_transfer64_kernel, G, T, 0, st, (int)nl, p->ib_face[a], (int)rows, p->K, p->fcol[a], p->fw64[a], p->ut64 + (long long)a * N, p->U64[a]);
