@@ -23,20 +23,20 @@ static int &ctas_ref(Plan *p, int axis, bool fp64) {
 static bool valid_ctas(int c) { return c == 1 || c == 2 || c == 4 || c == 8; }
 
 // Sweeps of the timed solve: a refined plan's first two, which is what the stopping rule mostly leaves.
-// Without them the 1024 x 512 channel's one-launch solve could lose to launches of variant 1, whose
-// transforms alone are about as fast; per projection these take 185 us against 129.
+// Without them the 1024 x 512 channel's one-launch solve (31 us for one solve) could lose to launches of
+// variant 1 (25), which take 185 us per projection against 129.
 static int tuned_sweeps(const Plan *p) {
   return p->precision == PC_PREC_MIXED ? (p->refine_iters < 2 ? p->refine_iters : 2) : 0;
 }
 
 // One solve of the plan's transform precision from s64 into the staging buffer.
-static pc_status run_solve(Plan *p, bool fp64, cudaStream_t st) {
+static pc_status run_solve(Plan *p, bool fp64, int sweeps, cudaStream_t st) {
   bool taken = false;
   if (fp64) {
     PC_TRY(solve_resident64(p, p->s64, p->stage_p, 0, st, taken));
     return taken ? PC_OK : solve_fp64_grid(p, p->s64, p->stage_p, st);
   }
-  if (tuned_sweeps(p) > 0) return solve_fixed_sweeps(p, p->s64, p->stage_p, tuned_sweeps(p), st);
+  if (sweeps > 0) return solve_fixed_sweeps(p, p->s64, p->stage_p, sweeps, st);
   // grids of the cooperative solve: one launch under the default schedule
   PC_TRY(solve_resident(p, p->s64, nullptr, p->stage_p, 0, false, 0.0f, grid_dev(p), st, taken));
   if (taken) return PC_OK;
@@ -44,13 +44,13 @@ static pc_status run_solve(Plan *p, bool fp64, cudaStream_t st) {
 }
 
 // Milliseconds per solve: two warm-up solves, then the best of three rounds of reps solves.
-static pc_status time_solve(Plan *p, bool fp64, cudaStream_t st, cudaEvent_t e0, cudaEvent_t e1, int reps,
+static pc_status time_solve(Plan *p, bool fp64, int sweeps, cudaStream_t st, cudaEvent_t e0, cudaEvent_t e1, int reps,
                             float &ms) {
-  for (int w = 0; w < 2; ++w) PC_TRY(run_solve(p, fp64, st));
+  for (int w = 0; w < 2; ++w) PC_TRY(run_solve(p, fp64, sweeps, st));
   ms = 1e30f;
   for (int round = 0; round < 3; ++round) {
     PC_CUDA_TRY(cudaEventRecord(e0, st));
-    for (int r = 0; r < reps; ++r) PC_TRY(run_solve(p, fp64, st));
+    for (int r = 0; r < reps; ++r) PC_TRY(run_solve(p, fp64, sweeps, st));
     PC_CUDA_TRY(cudaEventRecord(e1, st));
     PC_CUDA_TRY(cudaEventSynchronize(e1));
     float t = 0.0f;
@@ -70,11 +70,12 @@ static pc_status autotune(Plan *p, cudaStream_t st, double *best_out) {
   }
   pc_status status = PC_OK;
   float best = 0.0f;
-  const int reps = (p->ncells > (1 << 22) ? 3 : (p->ncells > (1 << 18) ? 12 : 30)) / (1 + tuned_sweeps(p));
+  const int sweeps = tuned_sweeps(p);
+  const int reps = (p->ncells > (1 << 22) ? 3 : (p->ncells > (1 << 18) ? 12 : 30)) / (1 + sweeps);
   if (cudaMemsetAsync(p->s64, 0, p->ncells * sizeof(double), st) != cudaSuccess ||
       cudaMemsetAsync(p->dstats, 0, sizeof(DevStats), st) != cudaSuccess)
     status = fail(PC_ERR_CUDA, "cudaMemsetAsync failed");
-  if (status == PC_OK) status = time_solve(p, fp64, st, e0, e1, reps, best);
+  if (status == PC_OK) status = time_solve(p, fp64, sweeps, st, e0, e1, reps, best);
   for (int round = 0; round < 2 && status == PC_OK; ++round) {
     bool changed = false;
     for (int a = 0; a < p->dim && status == PC_OK; ++a) {
@@ -88,7 +89,7 @@ static pc_status autotune(Plan *p, cudaStream_t st, double *best_out) {
           s = cand;
           if (fp64) p->ax[a].loop64 = false;
           float t = 0.0f;
-          const pc_status r = time_solve(p, fp64, st, e0, e1, reps, t);
+          const pc_status r = time_solve(p, fp64, sweeps, st, e0, e1, reps, t);
           if (r != PC_OK) {
             // a schedule the kernels cannot run (a tile too large): not a candidate
             cudaGetLastError();
@@ -108,6 +109,7 @@ static pc_status autotune(Plan *p, cudaStream_t st, double *best_out) {
     }
     if (!changed) break;
   }
+  if (status == PC_OK && sweeps > 0) status = time_solve(p, fp64, 0, st, e0, e1, reps, best);   // reported: one solve
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   plan_drop_graphs(p);
