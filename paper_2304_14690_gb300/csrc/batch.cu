@@ -264,7 +264,7 @@ pc_status record_exec(Exec *e, cudaStream_t st, Plan *prof = nullptr) {
   for (const Group &g : e->groups)
     for (int a = 0; a < g.dim; ++a) {
       const int n = (int)g.members.size();
-      batch_launch(BATCH_TRANSFER, g.sweeps ? g.K : -g.K, g.dP, segs(g, BATCH_TRANSFER + a), n, g.total[BATCH_TRANSFER + a], a, st);
+      batch_launch(BATCH_TRANSFER, 2 * g.K + (g.sweeps ? 0 : 1), g.dP, segs(g, BATCH_TRANSFER + a), n, g.total[BATCH_TRANSFER + a], a, st);
       ++launches;
     }
   mark(1);

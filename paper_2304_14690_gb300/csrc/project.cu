@@ -1383,15 +1383,17 @@ void batch_launch(int stage, int variant, const BatchProblem *P, const int *seg,
       if (variant == PC_DTYPE_F64) launch_pdl(batch_prep<double>, total_blocks, T, 0, st, P, seg, count);
       else launch_pdl(batch_prep<float>, total_blocks, T, 0, st, P, seg, count);
       break;
-    case BATCH_TRANSFER:   // variant: K, negative for unrefined plans
-      if (variant < 0) {   // the problems of a group share their sweeps: none
-        auto k = variant == -12 ? batch_transfer<12, true> : (variant == -27 ? batch_transfer<27, true> : batch_transfer<0, true>);
+    case BATCH_TRANSFER: {   // variant: 2 K, plus 1 for unrefined plans (the problems of a group share their sweeps)
+      const int K = variant >> 1;
+      if (variant & 1) {
+        auto k = K == 12 ? batch_transfer<12, true> : (K == 27 ? batch_transfer<27, true> : batch_transfer<0, true>);
         launch_pdl(k, total_blocks, T, 0, st, P, seg, count, extra);
       } else {
-        auto k = variant == 12 ? batch_transfer<12, false> : (variant == 27 ? batch_transfer<27, false> : batch_transfer<0, false>);
+        auto k = K == 12 ? batch_transfer<12, false> : (K == 27 ? batch_transfer<27, false> : batch_transfer<0, false>);
         launch_pdl(k, total_blocks, T, 0, st, P, seg, count, extra);
       }
       break;
+    }
     case BATCH_DIVERGENCE:   // variant: the group's dimension
       if (variant == 3) launch_pdl(batch_divergence<3>, total_blocks, T, 0, st, P, seg, count);
       else launch_pdl(batch_divergence<2>, total_blocks, T, 0, st, P, seg, count);
