@@ -313,6 +313,10 @@ struct Plan {
   long long launches = 0;
 };
 
+// Whether an FP32 solve of the plan is returned as the transforms round it (FP32 plans, and mixed ones
+// without sweeps): its fluxes and passes keep the steps, and so the bits, that such results always had.
+inline bool unrefined(const Plan *p) { return p->precision == PC_PREC_FP32 || p->refine_iters == 0; }
+
 // Profiler hooks (no-ops unless enabled): begin a call record, close the running segment as
 // phase `tag`, count kernel launches.
 void prof_begin(Plan *p, cudaStream_t st);

@@ -281,13 +281,13 @@ pc_status build_pass(const Plan *p, const PassSpec &ps, PassArgs<Real> &A, long 
   const bool lean = fp32 && deflt && pass_family(ax.kind) <= 2 && lean::length_ok(M) && quad &&
                     (E == 1 || !all || p->ncells > kResidentCells);
   const int lv = E == 1 ? 1 : 0;
-  // unrefined FP32 plans return the transforms' own rounding (1e-7): their bits stay those of the
+  // unrefined solves return the transforms' own rounding (1e-7): their bits stay those of the
   // general pass at the lengths without a compile-time one
-  const bool unrefined = fp32 && p->precision == PC_PREC_FP32 && !lean::length_ok(M);
+  const bool general = fp32 && unrefined(p) && !lean::length_ok(M);
   // FP64 lines of 4096 values leave one CTA per SM its shared memory for (4096 x 128: 229 us against
   // the general pass's 206; 2048 x 256: 160 against 238)
   const bool too_long = !fp32 && M > 1024;
-  if (deflt && !lean && quad && all && !unrefined && !too_long) {
+  if (deflt && !lean && quad && all && !general && !too_long) {
     // lines per tile: as many as the slots allow; a problem alone takes fewer where the GPU would
     // not be full (the lines do not depend on it)
     const int slots = fp32 ? kLoopSlots : kLoopSlots / 2;
@@ -550,7 +550,7 @@ pc_status solve_resident(Plan *p, const double *s64, const float2 *s2, double *p
   if (p->ncells > kResidentCells || sweeps > kMaxRefine) return PC_OK;
   for (int a = 0; a < p->dim; ++a) {
     if (p->ax[a].slots32 != 0 || p->ax[a].loop_nst == 0) return PC_OK;
-    if (p->precision == PC_PREC_FP32 && !lean::length_ok(p->ax[a].M)) return PC_OK;   // see build_pass
+    if (unrefined(p) && !lean::length_ok(p->ax[a].M)) return PC_OK;   // see build_pass
   }
   const void *rs = s2 ? (const void *)s2 : (const void *)s64;
   if (!aligned16(rs) || !aligned16(pout)) return PC_OK;

@@ -1591,8 +1591,6 @@ static void launch_residual(bool singular, bool write_r, bool norm, cudaStream_t
 // grid: no constant part in the DCT-I expansion), 2 zero first point. Problems with a zero mode
 // take the plan's gauge: the refinement cannot correct the constant that FP32 rounding leaves
 // (L_h of a constant is zero).
-static bool unrefined(const Plan *p) { return p->precision == PC_PREC_FP32 || p->refine_iters == 0; }
-
 // Fluxes of axis a: every face row, or the nl listed ones that an IB node reaches (nl >= 0).
 template <bool F64>
 static void launch_transfer(const Plan *p, int a, long long nl, cudaStream_t st) {

@@ -43,3 +43,24 @@ def test_batch_equals_single(pc, precision, iters, knn):
         assert all(torch.equal(x, y) for x, y in zip((a["p"], a["u"], a["f"]), want))
     for plan in plans:
         plan.close()
+
+
+# lengths with a compile-time pass (64, 256), without one (100, 200, 400, 40, 60), and both
+SOLVES = [((100, 200), "WP", "WP"), ((400, 400), "PP", "PP"), ((64, 200), "ID", "DW"), ((64, 256), "WW", "WW"),
+          ((40, 60, 100), "WPD", "WPW")]
+
+
+@pytest.mark.parametrize("n,lo,hi", SOLVES, ids=["x".join(map(str, s[0])) for s in SOLVES])
+def test_mixed_without_sweeps_is_the_fp32_solve(pc, n, lo, hi):
+    """A mixed plan without sweeps returns the bits of an FP32 plan: one solve and one projection."""
+    s = torch.randn(n, generator=torch.Generator(device="cuda").manual_seed(sum(n)), device="cuda", dtype=torch.float64)
+    q = wl.generic(dim=len(n), n=n, h=(1 / 64,) * len(n), bc_lo=lo, bc_hi=hi, seed=3)
+    u = torch.as_tensor(q.u_star, device="cuda")
+    got = []
+    for precision, iters in UNREFINED:
+        grid = pc.GridPlan(len(n), n, (1 / 64,) * len(n), lo, hi, precision=precision, refine_iters=iters)
+        plan = pc.Plan(q, precision=precision, refine_iters=iters)
+        got.append([grid.solve_poisson(s)[0].clone()] + [t.clone() for t in plan.project(u)[:3]])
+        grid.close()
+        plan.close()
+    assert all(torch.equal(a, b) for a, b in zip(*got))
