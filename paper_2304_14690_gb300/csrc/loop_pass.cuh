@@ -180,16 +180,17 @@ __device__ __forceinline__ void fft(const PassArgs<Real> &A, int L, int LS, type
       __syncthreads();
       continue;
     }
-    switch (si.R) {
-      case 16:
-        if constexpr (!SPLIT) stage<Real, 16>(a, b, L, LS, si, tb, p0);
-        break;
-      case 8: stage<Real, 8>(a, b, L, LS, si, tb, p0); break;
-      case 4: stage<Real, 4>(a, b, L, LS, si, tb, p0); break;
-      case 2: stage<Real, 2>(a, b, L, LS, si, tb, p0); break;
-      case 3: stage<Real, 3>(a, b, L, LS, si, tb, p0); break;
-      default: stage<Real, 5>(a, b, L, LS, si, tb, p0); break;
-    }
+    // Not a switch: with one, and an IEEE division elsewhere in the kernel, nvcc 13.0 let warps whose lanes
+    // end their loops at different iterations into the barrier in parts (a 60 x 720 solve off by 5e4,
+    // differently in each run). The warp barrier below is there for the same reason.
+    const int radix = si.R;
+    if (radix == 16) {
+      if constexpr (!SPLIT) stage<Real, 16>(a, b, L, LS, si, tb, p0);
+    } else if (radix == 8) stage<Real, 8>(a, b, L, LS, si, tb, p0);
+    else if (radix == 4) stage<Real, 4>(a, b, L, LS, si, tb, p0);
+    else if (radix == 2) stage<Real, 2>(a, b, L, LS, si, tb, p0);
+    else if (radix == 3) stage<Real, 3>(a, b, L, LS, si, tb, p0);
+    else stage<Real, 5>(a, b, L, LS, si, tb, p0);
     __syncthreads();
     T *t = a;
     a = b;
@@ -542,6 +543,7 @@ __device__ __forceinline__ void pass_tile(const PassArgs<Real> &A, int tile, typ
       if (fam == 0) divide_tile<Real, 0>(A, t, a, lam, tb);
       else if (fam == 1) divide_tile<Real, 1>(A, t, a, lam, tb);
       else divide_tile<Real, 2>(A, t, a, lam, tb);
+      __syncwarp();
       __syncthreads();
     }
   }
