@@ -5,7 +5,8 @@
 
 namespace pc {
 
-template <typename Real>
+// IEEE: for passes of which some divide with IEEE rounding (PassArgs::ieee_div).
+template <typename Real, bool IEEE>
 __global__ void __launch_bounds__(loop::kThreads, sizeof(Real) == 4 ? 4 : 2)
     loop_kernel(PassArgs<Real> A1, const PassArgs<Real> *__restrict__ args, const int4 *__restrict__ items) {
   pdl_enter();
@@ -34,28 +35,28 @@ __global__ void __launch_bounds__(loop::kThreads, sizeof(Real) == 4 ? 4 : 2)
   if (A.gate.st && refine_stopped_before(A.gate.st, A.gate.j, A.gate.tol)) return;   // refinement already ended
   for (int t = t0; t < t1; ++t) {
     if (t > t0) __syncthreads();   // the previous tile no longer reads the buffers
-    loop::pass_tile<Real, true>(A, t, buf, w16tab);
+    loop::pass_tile<Real, true, IEEE>(A, t, buf, w16tab);
   }
 }
 
 pc_status launch_loop(const PassArgs<float> &A, const PassArgs<float> *dargs, const int4 *ditems, unsigned grid,
-                      size_t smem, cudaStream_t st) {
+                      size_t smem, bool ieee, cudaStream_t st) {
   if (grid == 0) return PC_OK;
-  launch_pdl(loop_kernel<float>, grid, loop::kThreads, smem, st, A, dargs, ditems);
+  launch_pdl(ieee ? loop_kernel<float, true> : loop_kernel<float, false>, grid, loop::kThreads, smem, st, A, dargs, ditems);
   PC_CUDA_TRY(cudaGetLastError());
   return PC_OK;
 }
-pc_status launch_loop(const PassArgs<double> &A, const PassArgs<double> *dargs, const int4 *ditems, unsigned grid,
-                      size_t smem, cudaStream_t st) {
+pc_status launch_loop(const PassArgs<double> &A, unsigned grid, size_t smem, cudaStream_t st) {
   if (grid == 0) return PC_OK;
-  launch_pdl(loop_kernel<double>, grid, loop::kThreads, smem, st, A, dargs, ditems);
+  launch_pdl(loop_kernel<double, false>, grid, loop::kThreads, smem, st, A, (const PassArgs<double> *)nullptr, (const int4 *)nullptr);
   PC_CUDA_TRY(cudaGetLastError());
   return PC_OK;
 }
 
 pc_status prepare_loop(int lim) {
-  PC_CUDA_TRY(cudaFuncSetAttribute(loop_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
-  PC_CUDA_TRY(cudaFuncSetAttribute(loop_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
+  PC_CUDA_TRY(cudaFuncSetAttribute(loop_kernel<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
+  PC_CUDA_TRY(cudaFuncSetAttribute(loop_kernel<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
+  PC_CUDA_TRY(cudaFuncSetAttribute(loop_kernel<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
   return PC_OK;
 }
 

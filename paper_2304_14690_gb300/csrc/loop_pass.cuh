@@ -365,8 +365,17 @@ __device__ __forceinline__ void store_dst4(const Store<double> &A, int g, int st
   }
 }
 
-__device__ __forceinline__ float divide(float a, float b) { return __fdividef(a, b); }
-__device__ __forceinline__ double divide(double a, double b) { return a / b; }
+// Division by an eigenvalue sum. FP32: rounded to nearest where the axis's general pass did (A.ieee_div),
+// else the approximate one of the compile-time pass (2 ulp, and zero for divisors beyond 2^126), whose bits
+// this pass shares. IEEE: the kernel holds both; those without keep the registers of the approximate one.
+template <bool IEEE>
+__device__ __forceinline__ float divide(float a, float b, bool ieee) {
+  if constexpr (IEEE)
+    if (ieee) return __fdiv_rn(a, b);
+  return __fdividef(a, b);
+}
+template <bool IEEE>
+__device__ __forceinline__ double divide(double a, double b, bool) { return a / b; }
 
 // A tile in registers: line l (l < valid) starts at cell b0 + l * bstep and runs at `stride`.
 struct Tile {
@@ -433,12 +442,12 @@ __device__ __forceinline__ void fill_lambda(const PassArgs<Real> &A, const Tile 
 // Post-processing, division (the zero mode of a singular problem: coefficient 0 of the line at
 // cell 0) and pre-processing between the two halves of a dividing pass, pair by pair in registers,
 // in place.
-template <typename Real, int FAM, typename Tables>
+template <typename Real, int FAM, bool IEEE, typename Tables>
 __device__ __forceinline__ void divide_tile(const PassArgs<Real> &A, const Tile &t, typename Cplx<Real>::T *z,
                                             const Real *lam, const Tables &tb) {
   using T = typename Cplx<Real>::T;
   const int M = t.M, total = t.L * (M >> 1);
-  const bool dv = A.do_div, singular = A.singular && t.b0 == 0;
+  const bool dv = A.do_div, ieee = A.ieee_div, singular = A.singular && t.b0 == 0;
   for (int i = threadIdx.x; i < total; i += blockDim.x) {
     int l, k, qa, qb, pos[4];
     item_of(t, false, i, l, k);
@@ -452,7 +461,7 @@ __device__ __forceinline__ void divide_tile(const PassArgs<Real> &A, const Tile 
       const Real lo = lam[l];
 #pragma unroll
       for (int c = 0; c < 4; ++c)
-        val[c] = (singular && l == 0 && pos[c] == 0) ? (Real)0 : divide(val[c], tb.lam(pos[c]) + lo);
+        val[c] = (singular && l == 0 && pos[c] == 0) ? (Real)0 : divide<IEEE>(val[c], tb.lam(pos[c]) + lo, ieee);
     }
     T za, zb;
     inv_values<FAM>(val, M, k, t.kind, tb, za, zb);
@@ -511,7 +520,7 @@ __device__ __forceinline__ void load_coefs(const PassArgs<Real> &A, const Tile &
 // qd, stride) yields the input values at positions 4 qd .. 4 qd + 3 of line l (first cell base), and
 // put(l, base, qd, stride, x) takes the outputs of a final inverse. buf: two buffers of L lines, then the lines' eigenvalue sums. The two halves share one copy
 // of the FFT (a loop that is not unrolled). The caller puts a barrier before it; it ends without.
-template <typename Real, bool SPLIT, typename Tables, typename QuadFn, typename PutFn>
+template <typename Real, bool SPLIT, bool IEEE, typename Tables, typename QuadFn, typename PutFn>
 __device__ __forceinline__ void pass_tile(const PassArgs<Real> &A, int tile, typename Cplx<Real>::T *buf,
                                           const Tables &tb, const typename Cplx<Real>::T *w16tab, QuadFn quad, PutFn put) {
   using T = typename Cplx<Real>::T;
@@ -540,9 +549,9 @@ __device__ __forceinline__ void pass_tile(const PassArgs<Real> &A, int tile, typ
   for (int half = fwd ? 0 : 1; half < (inv ? 2 : 1); ++half) {
     fft<Real, SPLIT>(A, t.L, t.LS, a, b, tb, fam == 2 && half == 0 ? tw_dct4pre(M) : -1, w16tab);
     if (half == 0 && inv) {
-      if (fam == 0) divide_tile<Real, 0>(A, t, a, lam, tb);
-      else if (fam == 1) divide_tile<Real, 1>(A, t, a, lam, tb);
-      else divide_tile<Real, 2>(A, t, a, lam, tb);
+      if (fam == 0) divide_tile<Real, 0, IEEE>(A, t, a, lam, tb);
+      else if (fam == 1) divide_tile<Real, 1, IEEE>(A, t, a, lam, tb);
+      else divide_tile<Real, 2, IEEE>(A, t, a, lam, tb);
       __syncwarp();
       __syncthreads();
     }
@@ -569,14 +578,14 @@ __device__ __forceinline__ void pass_tile(const PassArgs<Real> &A, int tile, typ
 }
 
 // The pass on its plain source.
-template <typename Real, bool SPLIT>
+template <typename Real, bool SPLIT, bool IEEE>
 __device__ __forceinline__ void pass_tile(const PassArgs<Real> &A, int tile, typename Cplx<Real>::T *buf,
                                           const typename Cplx<Real>::T *w16tab) {
   const void *src = A.src;
   const int mode = A.src_mode;
   const GlobalTables<Real> tb{A.tw, A.stw, A.lam[A.axis]};
   const Store<Real> out = store_of(A);
-  pass_tile<Real, SPLIT>(
+  pass_tile<Real, SPLIT, IEEE>(
       A, tile, buf, tb, w16tab,
       [&](int, int base, int qd, int stride) { return load_src4<Real>(src, mode, base + 4 * qd * stride, stride); },
       [&](int, int base, int qd, int stride, const Quad<Real> &x) { store_dst4(out, base + 4 * qd * stride, stride, x); });

@@ -234,6 +234,7 @@ static long long fill_loop(const Plan *p, const PassSpec &ps, PassArgs<Real> &A,
   fill_pass<Real>(p, ps, A);
   A.loop = 1;
   A.fam = pass_family(ax.kind);
+  A.ieee_div = !lean::length_ok(ax.M);   // lengths with a compile-time pass keep its division, and its bits
   A.nst = ax.loop_nst;
   for (int s = 0; s < ax.loop_nst; ++s) A.st[s] = ax.loop_st[s];
   A.stw = A.tw + tw_total(ax.M);
@@ -389,7 +390,8 @@ static pc_status launch_pass(Plan *p, const PassSpec &ps, cudaStream_t st) {
   PC_TRY(build_pass<Real>(p, ps, A, tiles, threads, smem, 0));
   tiles = (tiles + A.chunk - 1) / A.chunk;   // CTAs
   if (A.loop) {
-    PC_TRY(launch_loop(A, nullptr, nullptr, (unsigned)tiles, smem, st));
+    if constexpr (sizeof(Real) == 4) PC_TRY(launch_loop(A, nullptr, nullptr, (unsigned)tiles, smem, A.do_div && A.ieee_div, st));
+    else PC_TRY(launch_loop(A, (unsigned)tiles, smem, st));
     count_launch(p);
     return PC_OK;
   }

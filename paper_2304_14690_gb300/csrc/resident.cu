@@ -158,7 +158,8 @@ __device__ __forceinline__ void cta_max(float v, float *dst) {
   }
 }
 
-template <int DIM, typename SV, bool CLUSTER>
+// IEEE: the pass of axis 0 divides with IEEE rounding (PassArgs::ieee_div).
+template <int DIM, typename SV, bool CLUSTER, bool IEEE>
 __global__ void __launch_bounds__(kResidentThreads, 1) resident_kernel(const __grid_constant__ ResidentArgs R) {
   constexpr int NP = 2 * DIM - 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -215,7 +216,7 @@ __global__ void __launch_bounds__(kResidentThreads, 1) resident_kernel(const __g
       for (int tile = t0; tile < t1; tile += step) {
         if (tile != t0) __syncthreads();   // the previous tile's outputs have left the buffers
         const int d0 = (tile - t0) * A.L;
-        loop::pass_tile<float, true>(
+        loop::pass_tile<float, true, IEEE>(
             A, tile, buf, tb, w16tab,
             [&](int l, int base, int qd, int stride) -> Quad<float> {
               if (!first) return loop::load_src4<float>(src, SRC_WORK, base + 4 * qd * stride, stride);
@@ -293,7 +294,7 @@ __global__ void __launch_bounds__(kResidentThreads, 1) resident_kernel(const __g
   }
 }
 
-template <int DIM, typename SV>
+template <int DIM, typename SV, bool IEEE>
 static pc_status launch(const ResidentArgs &R, size_t smem, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)R.grid);
@@ -310,33 +311,41 @@ static pc_status launch(const ResidentArgs &R, size_t smem, cudaStream_t st) {
     at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.numAttrs = tl_plain_launch ? 1 : 2;
-    PC_CUDA_TRY(cudaLaunchKernelEx(&cfg, resident_kernel<DIM, SV, true>, R));
+    PC_CUDA_TRY(cudaLaunchKernelEx(&cfg, resident_kernel<DIM, SV, true, IEEE>, R));
   } else {
     at[0].id = cudaLaunchAttributeCooperative;
     at[0].val.cooperative = 1;
     cfg.numAttrs = 1;
-    PC_CUDA_TRY(cudaLaunchKernelEx(&cfg, resident_kernel<DIM, SV, false>, R));
+    PC_CUDA_TRY(cudaLaunchKernelEx(&cfg, resident_kernel<DIM, SV, false, IEEE>, R));
   }
   return PC_OK;
 }
 
 pc_status launch_resident(const ResidentArgs &R, int dim, bool pairs, size_t smem, cudaStream_t st) {
-  if (dim == 2) return pairs ? launch<2, float2>(R, smem, st) : launch<2, double>(R, smem, st);
-  return pairs ? launch<3, float2>(R, smem, st) : launch<3, double>(R, smem, st);
+  auto of = [&](auto ieee) {
+    constexpr bool I = decltype(ieee)::value;
+    if (dim == 2) return pairs ? launch<2, float2, I>(R, smem, st) : launch<2, double, I>(R, smem, st);
+    return pairs ? launch<3, float2, I>(R, smem, st) : launch<3, double, I>(R, smem, st);
+  };
+  return R.pass[dim - 1].ieee_div ? of(std::true_type{}) : of(std::false_type{});
 }
 
-template <int DIM, typename SV>
+template <int DIM, typename SV, bool IEEE>
 static pc_status prepare_one() {
-  PC_CUDA_TRY(cudaFuncSetAttribute(resident_kernel<DIM, SV, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kResidentSmem));
-  PC_CUDA_TRY(cudaFuncSetAttribute(resident_kernel<DIM, SV, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kResidentSmem));
-  PC_CUDA_TRY(cudaFuncSetAttribute(resident_kernel<DIM, SV, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  PC_CUDA_TRY(cudaFuncSetAttribute(resident_kernel<DIM, SV, false, IEEE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kResidentSmem));
+  PC_CUDA_TRY(cudaFuncSetAttribute(resident_kernel<DIM, SV, true, IEEE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kResidentSmem));
+  PC_CUDA_TRY(cudaFuncSetAttribute(resident_kernel<DIM, SV, true, IEEE>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   return PC_OK;
 }
 pc_status prepare_resident() {
-  PC_TRY((prepare_one<2, float2>()));
-  PC_TRY((prepare_one<2, double>()));
-  PC_TRY((prepare_one<3, float2>()));
-  return prepare_one<3, double>();
+  PC_TRY((prepare_one<2, float2, false>()));
+  PC_TRY((prepare_one<2, float2, true>()));
+  PC_TRY((prepare_one<2, double, false>()));
+  PC_TRY((prepare_one<2, double, true>()));
+  PC_TRY((prepare_one<3, float2, false>()));
+  PC_TRY((prepare_one<3, float2, true>()));
+  PC_TRY((prepare_one<3, double, false>()));
+  return prepare_one<3, double, true>();
 }
 
 int resident_cluster_size() {
@@ -354,7 +363,7 @@ int resident_cluster_size() {
       at[0].val.clusterDim.x = (unsigned)n;
       cfg.gridDim = dim3((unsigned)n);
       int fit = 0;
-      if (cudaOccupancyMaxActiveClusters(&fit, resident_kernel<3, double, true>, &cfg) == cudaSuccess && fit > 0) return n;
+      if (cudaOccupancyMaxActiveClusters(&fit, resident_kernel<3, double, true, true>, &cfg) == cudaSuccess && fit > 0) return n;
       cudaGetLastError();
     }
     return 0;
