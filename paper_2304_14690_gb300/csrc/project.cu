@@ -486,38 +486,32 @@ __device__ __forceinline__ double trap_weight(const TrapWeights &w, long long c)
 }
 
 // Sum (weighted, see TrapWeights) of a cell array (the source of pc_solve_poisson) and its mean;
-// SQUARES: also the sum of squares (statistics). Mixed plans, whose refinement reads the mean on
-// every call, sum in double-float arithmetic (both sums in FP64 took 59 us on a 192^3 grid, on the
-// FP64 pipe); the others need the sums for statistics alone and take FP64.
-template <bool MIXED, bool SQUARES>
+// SQUARES: also the sum of squares (statistics).
+template <bool SQUARES>
 __device__ __forceinline__ void sum_kernel_body(unsigned b, unsigned nblk, long long count, const double *x,
                                                 DevStats *stats, double *partials, unsigned int *counter,
                                                 const TrapWeights &w) {
-  DF d1{0.0f, 0.0f};
   double v1 = 0.0, v2 = 0.0;
 #pragma unroll
   for (int k = 0; k < kFlatPerThread; ++k) {
     const long long c = (long long)b * kFlatPerBlock + k * kFlatThreads + threadIdx.x;
     if (c < count) {
       const double v = x[c];
-      const double wv = w.dim ? trap_weight(w, c) * v : v;   // a power of two: exact
-      if (MIXED) d1 = df_add(d1, df_of(wv));
-      else v1 += wv;
+      v1 += w.dim ? trap_weight(w, c) * v : v;
       if (SQUARES) v2 = fma(v, v, v2);
     }
   }
   const VBlock vb{b, 0u, 0u, nblk, 1u, 1u};
-  if (MIXED) v1 = f2d_bits(d1.hi) + f2d_bits(d1.lo);
   if (grid_sum(v1, partials, counter, &stats->sum_s, vb))
     stats->mean_s = stats->sum_s / (w.dim ? w.total : (double)count);
   if (SQUARES) grid_sum(v2, partials + nblk, counter + 1, &stats->sum_s2, vb);
 }
 
-template <bool MIXED, bool SQUARES>
+template <bool SQUARES>
 __global__ void sum_kernel(long long count, const double *x, DevStats *stats, double *partials,
                            unsigned int *counter, TrapWeights w) {
   pdl_enter();
-  sum_kernel_body<MIXED, SQUARES>(blockIdx.x, gridDim.x, count, x, stats, partials, counter, w);
+  sum_kernel_body<SQUARES>(blockIdx.x, gridDim.x, count, x, stats, partials, counter, w);
 }
 
 // ----------------------------------------------------------------------------- residual
@@ -1610,11 +1604,6 @@ static void launch_transfer(const Plan *p, int a, long long nl, cudaStream_t st)
 // transforms themselves drop the zero mode.
 static bool needs_mean(const Plan *p) { return p->singular && p->precision == PC_PREC_MIXED && p->refine_iters > 0; }
 
-static auto sum_kernel_of(const Plan *p, bool squares) {
-  if (p->precision == PC_PREC_MIXED) return squares ? sum_kernel<true, true> : sum_kernel<true, false>;
-  return squares ? sum_kernel<false, true> : sum_kernel<false, false>;
-}
-
 static int gauge_mode(const Plan *p) {
   if (!p->singular) return 0;
   return p->gauge == 1 ? 2 : 1;
@@ -1852,7 +1841,7 @@ static pc_status vertex_pass_solve(Plan *p, cudaStream_t st, double inv_bdt, dou
   // the source sums: the (weighted) mean the residual removes on zero-mode problems, and the
   // statistics
   if (want_stats || needs_mean(p)) {
-    launch_pdl(sum_kernel_of(p, want_stats), grid_for(nc, kFlatPerBlock), kFlatThreads, 0, st, nc, (const double *)p->s64, p->dstats,
+    launch_pdl(want_stats ? sum_kernel<true> : sum_kernel<false>, grid_for(nc, kFlatPerBlock), kFlatThreads, 0, st, nc, (const double *)p->s64, p->dstats,
                p->partials, p->counters, trap_weights(p));
     count_launch(p);
   }
@@ -2021,7 +2010,7 @@ static pc_status vertex_solve(Plan *p, const double *s, double *p_out, pc_stats 
   prof_begin(p, st);
   PC_CUDA_TRY(cudaMemsetAsync(p->dstats, 0, sizeof(DevStats), st));
   if (needs_mean(p) || stats) {
-    launch_pdl(sum_kernel_of(p, stats != nullptr), grid_for(nc, kFlatPerBlock), kFlatThreads, 0, st, nc, ds, p->dstats, p->partials,
+    launch_pdl(stats ? sum_kernel<true> : sum_kernel<false>, grid_for(nc, kFlatPerBlock), kFlatThreads, 0, st, nc, ds, p->dstats, p->partials,
                p->counters, trap_weights(p));
     count_launch(p);
   }
@@ -2045,7 +2034,7 @@ static pc_status solve_impl(Plan *p, const double *s, double *p_out, pc_stats *s
   prof_begin(p, st);
   PC_CUDA_TRY(cudaMemsetAsync(p->dstats, 0, sizeof(DevStats), st));
   if (needs_mean(p) || stats) {
-    launch_pdl(sum_kernel_of(p, stats != nullptr), grid_for(nc, kFlatPerBlock), kFlatThreads, 0, st, nc, ds, p->dstats, p->partials, p->counters,
+    launch_pdl(stats ? sum_kernel<true> : sum_kernel<false>, grid_for(nc, kFlatPerBlock), kFlatThreads, 0, st, nc, ds, p->dstats, p->partials, p->counters,
                TrapWeights{});
     count_launch(p);
   }

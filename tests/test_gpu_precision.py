@@ -35,3 +35,18 @@ def test_division_by_large_eigenvalues(pc, n, lo, hi):
         p[precision] = plan.solve_poisson(s)[0].clone()
         plan.close()
     assert float((p["mixed"] - p["fp64"]).norm() / p["fp64"].norm()) <= 1e-10
+
+
+def test_mean_of_the_source_in_64_bits(pc):
+    """The mean of 1 + r and 1 - r in rows of four, r = 2^-24 + 15 * 2^-51, on 64 x 64 cells. A thread of
+    the sum takes cells 256 apart, two of each: in FP64 its sums are exact (r is a multiple of 2^-51,
+    and 3 + r has 53 bits), and all that follow add fours. As FP32 pairs both values lose their last
+    bits, in the same direction."""
+    r = 2.0 ** -24 + 15 * 2.0 ** -51
+    s = torch.ones((64, 64), dtype=torch.float64, device="cuda")
+    up = (torch.arange(64, device="cuda") // 4) % 2 == 0
+    s[up] += r
+    s[~up] -= r
+    plan = pc.GridPlan(2, (64, 64), (1 / 64, 1 / 64), "WW", "WW", precision="mixed")
+    assert plan.solve_poisson(s, stats=True)[1]["removed_mean"] == 1.0
+    plan.close()
