@@ -394,8 +394,9 @@ pc_status pc_set_graphs(pc_plan *plan, int on);
  * looped passes, larger grids the compile-time pass of the axis's line length where it has one
  * (n = 2M with M in {16, 32, 48, 64, 96, 128, 192, 256, 384, 512}), with the same bits; axes without
  * either take 4 slots. With 1: the compile-time pass with fewer slots and more threads per line.
- * FP64 passes with M <= 1024 take the looped passes (small grids one kernel) until a slot count is
- * set or the autotuner finds a faster one.
+ * FP64 passes take slots = 2, the default, as the looped passes where every axis has them (even
+ * M = n/2, cell grids) and M <= 1024, with 2 on every axis up to about a million cells as one kernel.
+ * What pc_plan_get_transform_slots returns can be set again, on this plan or another of the grid.
  * Errors: PC_ERR_INVALID_ARG for a bad axis or slot count; a schedule whose tile does not fit the
  * kernels fails at the next call with PC_ERR_UNSUPPORTED. Defaults: 0 (FP32), 2 (FP64). */
 pc_status pc_plan_set_transform_slots(pc_plan *plan, int axis, pc_precision precision, int slots);

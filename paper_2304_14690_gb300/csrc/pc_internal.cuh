@@ -60,8 +60,6 @@ struct AxisInfo {
   // twiddles follow the tables above in both precisions.
   int loop_nst = 0;
   StageInfo loop_st[kMaxRadices];
-  // FP64 passes: the looped ones until a slot count is set or the autotuner finds a faster one
-  bool loop64 = true;
   double *lam64 = nullptr;   // eigenvalue per spectral index (n entries)
   float *lam32 = nullptr;
 };

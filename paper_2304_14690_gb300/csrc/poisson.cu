@@ -268,10 +268,11 @@ pc_status build_pass(const Plan *p, const PassSpec &ps, PassArgs<Real> &A, long 
   const AxisInfo &ax = p->ax[axis];
   const int M = ax.M;
   // slots per thread; 0 and 1 (FP32 only): variant 0 or 1 of the lean pass of the length
-  // (lean_pass.cuh) where it has one, else the looped pass (loop_pass.cuh) where it has one, else 4
+  // (lean_pass.cuh) where it has one, else the looped pass (loop_pass.cuh) where it has one, else 4;
+  // FP64: 2, the default, the looped pass where the axis has one
   const bool fp32 = sizeof(Real) == 4;
   int E = fp32 ? ax.slots32 : ax.slots64;
-  const bool deflt = fp32 ? E <= 1 : ax.loop64;
+  const bool deflt = fp32 ? E <= 1 : E == 2;
   const bool quad = quad_io(p, ps, fp32);
   bool all = true;   // an axis without a looped pass (odd M, vertex kinds): none on the others either
   for (int a = 0; a < p->dim; ++a) all = all && p->ax[a].loop_nst > 0;
@@ -589,7 +590,7 @@ pc_status solve_resident64(Plan *p, const double *s, double *pout, int gauge, cu
   taken = false;
   if (p->ncells > kResident64Cells || !aligned16(s) || !aligned16(pout)) return PC_OK;
   for (int a = 0; a < p->dim; ++a)
-    if (!p->ax[a].loop64 || p->ax[a].loop_nst == 0 || p->ax[a].M > 1024) return PC_OK;
+    if (p->ax[a].slots64 != 2 || p->ax[a].loop_nst == 0 || p->ax[a].M > 1024) return PC_OK;
   Resident64Args R;
   memset(&R, 0, sizeof(R));
   R.cluster = p->ncells <= kCluster64Cells && resident_cluster_size() > 0;

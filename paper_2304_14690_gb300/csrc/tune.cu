@@ -83,18 +83,15 @@ static pc_status autotune(Plan *p, cudaStream_t st, double *best_out) {
       for (int knob = 0; knob < 2; ++knob) {
         int &s = knob == 0 ? slots_ref(p, a, fp64) : ctas_ref(p, a, fp64);
         for (int cand : {0, 1, 2, 4, 8, 16}) {
-          if ((cand == s && !(fp64 && knob == 0 && p->ax[a].loop64)) || (knob == 0 ? !valid_slots(cand, fp64) : !valid_ctas(cand))) continue;
+          if (cand == s || (knob == 0 ? !valid_slots(cand, fp64) : !valid_ctas(cand))) continue;
           const int keep = s;
-          const bool keep_loop = p->ax[a].loop64;
           s = cand;
-          if (fp64) p->ax[a].loop64 = false;
           float t = 0.0f;
           const pc_status r = time_solve(p, fp64, sweeps, st, e0, e1, reps, t);
           if (r != PC_OK) {
             // a schedule the kernels cannot run (a tile too large): not a candidate
             cudaGetLastError();
             s = keep;
-            p->ax[a].loop64 = keep_loop;
             continue;
           }
           if (t < 0.98f * best) {
@@ -102,7 +99,6 @@ static pc_status autotune(Plan *p, cudaStream_t st, double *best_out) {
             changed = true;
           } else {
             s = keep;
-            p->ax[a].loop64 = keep_loop;
           }
         }
       }
@@ -126,7 +122,6 @@ extern "C" pc_status pc_plan_set_transform_slots(pc_plan *plan, int axis, pc_pre
   if (!pc::valid_slots(slots, precision == PC_PREC_FP64))
     return pc::fail(PC_ERR_INVALID_ARG, "slots must be 2, 4, 8 or 16, or 0 or 1 for FP32 (got %d)", slots);
   pc::slots_ref(p, axis, precision == PC_PREC_FP64) = slots;
-  if (precision == PC_PREC_FP64) p->ax[axis].loop64 = false;
   pc::plan_drop_graphs(p);
   return PC_OK;
 }
