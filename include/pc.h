@@ -404,7 +404,8 @@ pc_status pc_plan_get_transform_slots(const pc_plan *plan, int axis, pc_precisio
                                       int *slots_out);
 
 /* Tile size of the single-problem passes along `axis`: the number of lines per CTA is halved
- * until the pass has at least ctas_per_sm x 152 CTAs (1, 2, 4 or 8; default 2). Part of the
+ * until the pass has at least ctas_per_sm x 152 CTAs (1, 2, 4 or 8; default 2). The general passes
+ * alone take it: the looped, one-launch and compile-time ones size their own tiles. Part of the
  * schedule like the slots: it drops the plan's graphs, leaves batched calls (whose tiles fill a
  * fixed CTA) alone, and does not change results (each line is transformed the same way in any
  * tile). Errors: PC_ERR_INVALID_ARG for a bad axis or count. */

@@ -29,6 +29,24 @@ static int tuned_sweeps(const Plan *p) {
   return p->precision == PC_PREC_MIXED ? (p->refine_iters < 2 ? p->refine_iters : 2) : 0;
 }
 
+// Whether a pass along the axis is a general one under the current schedule: the CTA target sizes no others.
+static bool has_general_pass(const Plan *p, int axis, bool fp64) {
+  for (const PassSpec &ps : solve_pass_specs(p, !fp64, SRC_F64, p->s64, DST_F64_SET, p->stage_p)) {
+    if (ps.axis != axis) continue;
+    long long tiles;
+    int threads;
+    size_t smem;
+    if (fp64) {
+      PassArgs<double> A;
+      if (build_pass<double>(p, ps, A, tiles, threads, smem, 0) == PC_OK && !A.loop) return true;
+    } else {
+      PassArgs<float> A;
+      if (build_pass<float>(p, ps, A, tiles, threads, smem, 0) == PC_OK && !A.loop && !A.lean) return true;
+    }
+  }
+  return false;
+}
+
 // One solve of the plan's transform precision from s64 into the staging buffer.
 static pc_status run_solve(Plan *p, bool fp64, int sweeps, cudaStream_t st) {
   bool taken = false;
@@ -81,6 +99,7 @@ static pc_status autotune(Plan *p, cudaStream_t st, double *best_out) {
     for (int a = 0; a < p->dim && status == PC_OK; ++a) {
       // the two knobs of the axis in turn: slots per thread, then CTAs per SM
       for (int knob = 0; knob < 2; ++knob) {
+        if (knob == 1 && !has_general_pass(p, a, fp64)) continue;
         int &s = knob == 0 ? slots_ref(p, a, fp64) : ctas_ref(p, a, fp64);
         for (int cand : {0, 1, 2, 4, 8, 16}) {
           if (cand == s || (knob == 0 ? !valid_slots(cand, fp64) : !valid_ctas(cand))) continue;
