@@ -381,6 +381,9 @@ pc_status solve_fp64_grid(Plan *p, const double *s, double *pout, cudaStream_t s
 pc_status solve_fp32_grid(Plan *p, int src_mode, const void *s, int dst_mode, void *dst,
                           cudaStream_t st, double *f64 = nullptr, RefineGate gate = RefineGate{nullptr, 0, 0.0f},
                           int chunk = 1);
+// Largest grid of the cooperative solve: what the SMs' shared memory holds (1024^2: 135 us against
+// 258 by launches); the fit itself is checked for each plan.
+constexpr long long kResidentCells = 1LL << 20;
 // Geometry of a plan's pressure grid for the cell kernels (project.cu).
 GridDev grid_dev(const Plan *p);
 // The refined FP32 solve as one cooperative kernel (resident.cu) where the plan and the arrays allow

@@ -243,9 +243,6 @@ static long long fill_loop(const Plan *p, const PassSpec &ps, PassArgs<Real> &A,
   return fill_tiles<Real>(p, A, L);
 }
 
-// Largest grid of the cooperative solve: what the SMs' shared memory holds (1024^2: 135 us against
-// 258 by launches); the fit itself is checked for each plan.
-constexpr long long kResidentCells = 1LL << 20;
 // Slots of a looped pass's tile: 2048 in FP32 (35 KB: six CTAs of 256 threads per SM) and 1024 in
 // FP64 in a launch of its own (4096: 64 2D problems 868 us against 823), up to 4096 on the resident CTAs.
 constexpr int kLoopSlots = 2048;
