@@ -420,6 +420,14 @@ pc_status pc_plan_get_transform_ctas(const pc_plan *plan, int axis, pc_precision
  * during a stream capture or while a call of the plan is in flight. */
 pc_status pc_plan_autotune(pc_plan *plan, void *cuda_stream, double *best_ms_out);
 
+/* Most polls of one wait inside the plan's solves (default 2^22, about two seconds). Solves of up to
+ * about a million cells may run as one kernel whose thread blocks wait for one another; where a wait
+ * runs out, the kernel ends, the pressure (and what follows from it) holds NaN, and PC_ERR_TIMEOUT is
+ * returned: by the same call if it waits for the device (statistics, host arrays, pc_project_ib,
+ * pc_plan_autotune), else by the next call on the plan, which then does nothing else. The plan stays
+ * usable. 0: solves take one launch per pass and nothing waits. Drops the plan's captured graphs. */
+pc_status pc_plan_set_wait_limit(pc_plan *plan, unsigned int polls);
+
 /* Device bytes held by the plan. */
 pc_status pc_plan_bytes(const pc_plan *plan, size_t *bytes_out);
 

@@ -104,6 +104,11 @@ void plan_drop_graphs(Plan *p) {
   }
 }
 
+pc_status wait_status(Plan *p) {
+  if (!p->gave_up || !__atomic_exchange_n(p->gave_up, 0u, __ATOMIC_ACQ_REL)) return PC_OK;
+  return fail(PC_ERR_TIMEOUT, "a wait inside a solve of this plan gave up: its pressure holds NaN");
+}
+
 static void destroy_plan(Plan *p) {
   if (!p) return;
   batch_forget_plan(p);
@@ -124,6 +129,7 @@ static void destroy_plan(Plan *p) {
     if (p->copy_ev[e]) cudaEventDestroy(p->copy_ev[e]);
   if (p->ib_body_stream) cudaStreamDestroy(p->ib_body_stream);
   for (int i = 0; i < p->nallocs; ++i) cudaFree(p->allocs[i]);
+  if (p->gave_up) cudaFreeHost(p->gave_up);
   if (cur >= 0) cudaSetDevice(cur);
   delete p;
 }
@@ -213,6 +219,9 @@ static pc_status alloc_workspace(Plan *p, cudaStream_t st) {
   if (cudaMemsetAsync(p->counters, 0, 16 * sizeof(unsigned int), st) != cudaSuccess ||
       cudaMemsetAsync(p->dstats, 0, sizeof(DevStats), st) != cudaSuccess)
     return fail(PC_ERR_CUDA, "counter reset failed");
+  if (cudaHostAlloc((void **)&p->gave_up, sizeof(unsigned), cudaHostAllocPortable) != cudaSuccess)
+    return fail(PC_ERR_CUDA, "host word allocation failed");
+  *p->gave_up = 0u;
   if (cudaStreamCreateWithFlags(&p->cap_stream, cudaStreamNonBlocking) != cudaSuccess)
     return fail(PC_ERR_CUDA, "stream creation failed");
   for (int e = 0; e < kProfEvents; ++e)
@@ -609,6 +618,7 @@ extern "C" pc_status pc_plan_clone(pc_plan *plan, void *cuda_stream, pc_plan **o
   p->divmode = root->divmode; p->ccol = root->ccol; p->cD64 = root->cD64; p->cD2 = root->cD2;
   p->ncol = root->ncol; p->nD64 = root->nD64; p->nD2 = root->nD2; p->ntype = root->ntype;
   p->graphs_on = root->graphs_on;
+  p->wait_polls = root->wait_polls;
   p->vertex = root->vertex; p->problem_singular = root->problem_singular;
   p->nvtot = root->nvtot; p->nftot = root->nftot; p->npts = root->npts;
   for (int a = 0; a < 3; ++a) { p->phys_L[a] = root->phys_L[a]; p->phys_periodic[a] = root->phys_periodic[a]; }
@@ -675,6 +685,16 @@ extern "C" pc_status pc_set_graphs(pc_plan *plan, int on) {
   pc::Plan *p = reinterpret_cast<pc::Plan *>(plan);
   if (!p) return pc::fail(PC_ERR_INVALID_ARG, "plan is NULL");
   p->graphs_on = on != 0;
+  return PC_OK;
+}
+
+extern "C" pc_status pc_plan_set_wait_limit(pc_plan *plan, unsigned int polls) {
+  pc::Plan *p = reinterpret_cast<pc::Plan *>(plan);
+  if (!p) return pc::fail(PC_ERR_INVALID_ARG, "plan is NULL");
+  if (polls != p->wait_polls) {
+    p->wait_polls = polls;
+    pc::plan_drop_graphs(p);   // captured launches hold the limit
+  }
   return PC_OK;
 }
 

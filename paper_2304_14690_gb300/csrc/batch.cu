@@ -430,6 +430,7 @@ pc_status validate_batch(int count, pc_plan *const *plans, const pc_project_args
       }
     }
   }
+  for (int i = 0; i < count; ++i) PC_TRY(wait_status(reinterpret_cast<Plan *>(plans[i])));
   return PC_OK;
 }
 

@@ -23,7 +23,7 @@ constexpr long long kMaxRows = (1LL << 31) - (1LL << 16);
 constexpr int kMaxRefine = 8;
 
 // Device-side status word values (written by kernels, read at the next sync point).
-enum DeviceFlag { FLAG_WLS_SINGULAR = 1, FLAG_KNN_SHORT = 2, FLAG_NONFINITE = 4, FLAG_TIMEOUT = 8 };
+enum DeviceFlag { FLAG_WLS_SINGULAR = 1, FLAG_KNN_SHORT = 2, FLAG_NONFINITE = 4 };
 
 // One FFT stage: radix R, current span Ns, twiddle stride M/(Ns R). j / Ns is a shift when Ns
 // is a power of two, else a multiply-high by magic = ceil(2^32/Ns) (exact for j < 2^16).
@@ -246,6 +246,10 @@ struct Plan {
   DevStats *dstats = nullptr;
   double *partials = nullptr;      // per-block partial sums of the deterministic reductions
   unsigned int *counters = nullptr;  // completion counters of those reductions (kept at zero)
+  // one-launch solves (resident.cu): polls of one grid barrier at most (about two seconds; 0: solves take
+  // one launch per pass), and the pinned host word they set where one gave up
+  unsigned wait_polls = 1u << 22;
+  unsigned *gave_up = nullptr;
   // Staging for host pointers passed to pc_project.
   void *stage_u = nullptr, *stage_f = nullptr, *stage_uo = nullptr, *stage_fo = nullptr;
   // copy stream and events of the host-array path (results copied back while kernels run)
@@ -394,6 +398,8 @@ pc_status solve_resident(Plan *p, const double *s64, const float2 *s2, double *p
                          float tol, const GridDev &g, cudaStream_t st, bool &taken);
 // The plain FP64 solve of a small grid with its gauge (gauge_mode) as one launch (resident64.cu).
 pc_status solve_resident64(Plan *p, const double *s, double *pout, int gauge, cudaStream_t st, bool &taken);
+// PC_ERR_TIMEOUT if a barrier of the plan's solves has given up since the last call that said so.
+pc_status wait_status(Plan *p);
 // Drops the plan's captured CUDA graphs and batch executables (after a schedule change).
 void plan_drop_graphs(Plan *p);
 // ----------------------------------------------------------------------------- batches

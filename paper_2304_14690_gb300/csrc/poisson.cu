@@ -547,7 +547,7 @@ static int sm_count() {
 pc_status solve_resident(Plan *p, const double *s64, const float2 *s2, double *pout, int sweeps, bool adaptive,
                          float tol, const GridDev &g, cudaStream_t st, bool &taken) {
   taken = false;
-  if (p->ncells > kResidentCells || sweeps > kMaxRefine) return PC_OK;
+  if (p->wait_polls == 0 || p->ncells > kResidentCells || sweeps > kMaxRefine) return PC_OK;
   for (int a = 0; a < p->dim; ++a) {
     if (p->ax[a].slots32 != 0 || p->ax[a].loop_nst == 0) return PC_OK;
     if (unrefined(p) && !lean::length_ok(p->ax[a].M)) return PC_OK;   // see build_pass
@@ -572,6 +572,8 @@ pc_status solve_resident(Plan *p, const double *s64, const float2 *s2, double *p
   R.adaptive = adaptive;
   R.singular = p->singular;
   R.tol = tol;
+  R.polls = p->wait_polls;
+  R.gave_up = p->gave_up;
   PC_TRY(launch_resident(R, p->dim, s2 != nullptr, smem, st));
   count_launch(p);
   taken = true;
@@ -585,7 +587,7 @@ constexpr long long kResident64Cells = 1LL << 20, kCluster64Cells = 4096;
 
 pc_status solve_resident64(Plan *p, const double *s, double *pout, int gauge, cudaStream_t st, bool &taken) {
   taken = false;
-  if (p->ncells > kResident64Cells || !aligned16(s) || !aligned16(pout)) return PC_OK;
+  if (p->wait_polls == 0 || p->ncells > kResident64Cells || !aligned16(s) || !aligned16(pout)) return PC_OK;
   for (int a = 0; a < p->dim; ++a)
     if (p->ax[a].slots64 != 2 || p->ax[a].loop_nst == 0 || p->ax[a].M > 1024) return PC_OK;
   Resident64Args R;
@@ -604,6 +606,8 @@ pc_status solve_resident64(Plan *p, const double *s, double *pout, int gauge, cu
   R.bar = p->dstats->bar;
   R.gauge = gauge;
   R.inv_cells = 1.0 / (double)p->ncells;
+  R.polls = p->wait_polls;
+  R.gave_up = p->gave_up;
   PC_TRY(launch_resident64(R, p->dim, smem, st));
   count_launch(p);
   taken = true;

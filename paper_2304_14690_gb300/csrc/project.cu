@@ -1724,6 +1724,7 @@ static pc_status fill_stats(Plan *p, pc_stats *stats, cudaStream_t st) {
   PC_CUDA_TRY(cudaMemcpyAsync(&ds, p->dstats, sizeof(DevStats), cudaMemcpyDeviceToHost, st));
   PC_CUDA_TRY(cudaStreamSynchronize(st));
   memset(stats, 0, sizeof(*stats));
+  PC_TRY(wait_status(p));
   const double nc = mean_weight_total(p);   // cells, or the trapezoid weights of a vertex grid
   const bool zero_mode = p->singular;
   stats->removed_mean = zero_mode ? ds.sum_s / nc : 0.0;
@@ -1983,8 +1984,9 @@ static pc_status project_impl(Plan *p, double dt, const void *u_star, const void
     PC_CUDA_TRY(cudaStreamWaitEvent(st, p->copy_ev[2], 0));
   }
   if (stats) PC_TRY(fill_stats(p, stats, st));
-  if (hp || huo || (f_out && hfo)) PC_CUDA_TRY(cudaStreamSynchronize(st));
-  return PC_OK;
+  if (!(hp || huo || (f_out && hfo))) return PC_OK;
+  PC_CUDA_TRY(cudaStreamSynchronize(st));
+  return wait_status(p);
 }
 
 // Grid-level solve of device arrays with a caller-built plan description (FP64; no staging, no
@@ -2042,8 +2044,9 @@ static pc_status solve_impl(Plan *p, const double *s, double *p_out, pc_stats *s
   PC_TRY(solve_grid(p, ds, dp, stats != nullptr, st));
   if (hp) PC_CUDA_TRY(cudaMemcpyAsync(p_out, dp, nc * sizeof(double), cudaMemcpyDeviceToHost, st));
   if (stats) PC_TRY(fill_stats(p, stats, st));
-  if (hp) PC_CUDA_TRY(cudaStreamSynchronize(st));
-  return PC_OK;
+  if (!hp) return PC_OK;
+  PC_CUDA_TRY(cudaStreamSynchronize(st));
+  return wait_status(p);
 }
 
 static bool graph_cached(const Plan *p, double dt, const void *u, const void *f, const double *po,
@@ -2465,6 +2468,7 @@ static pc_status project_ib_impl(Plan *p, double dt, const VT *du, const VT *f_i
                                 cudaMemcpyDeviceToHost, st));
     PC_CUDA_TRY(cudaStreamSynchronize(st));
   }
+  PC_TRY(wait_status(p));
   if (history)
     for (int k = 0; k < h.it; ++k) { history[2 * k] = h.hist[2 * k]; history[2 * k + 1] = h.hist[2 * k + 1]; }
   if (res) {
@@ -2490,6 +2494,7 @@ extern "C" pc_status pc_project(pc_plan *plan, double dt, const void *u_star, co
   if (p->grid_only) return pc::fail(PC_ERR_INVALID_ARG, "a grid-only plan has no nodes: use pc_solve_poisson");
   if (!u_star || !p_out || !u_out) return pc::fail(PC_ERR_INVALID_ARG, "u_star, p_out and u_out are required");
   if (!(dt > 0.0) || !std::isfinite(dt)) return pc::fail(PC_ERR_INVALID_ARG, "dt must be positive and finite");
+  PC_TRY(pc::wait_status(p));
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev != p->device) {
     if (cudaSetDevice(p->device) != cudaSuccess) return pc::fail(PC_ERR_CUDA, "cannot select device %d", p->device);
@@ -2506,6 +2511,7 @@ extern "C" pc_status pc_solve_poisson(pc_plan *plan, const double *s, double *p_
                                       void *cuda_stream) {
   pc::Plan *p = reinterpret_cast<pc::Plan *>(plan);
   if (!p || !s || !p_out) return pc::fail(PC_ERR_INVALID_ARG, "plan, s and p_out are required");
+  PC_TRY(pc::wait_status(p));
   if (cudaSetDevice(p->device) != cudaSuccess) return pc::fail(PC_ERR_CUDA, "cannot select device %d", p->device);
   // device arrays without statistics: one launch of a graph cached per (s, p_out)
   if (p->graphs_on && !stats && pc::is_device_ptr(s) && pc::is_device_ptr(p_out))
@@ -2525,6 +2531,7 @@ extern "C" pc_status pc_project_ib(pc_plan *plan, double dt, const void *u_star,
   if (!(tol >= 0.0) || !std::isfinite(tol)) return pc::fail(PC_ERR_INVALID_ARG, "tol must be finite and >= 0");
   if (max_iters < 1 || max_iters > pc::kIbMaxIters)
     return pc::fail(PC_ERR_INVALID_ARG, "max_iters must be in [1, %d]", pc::kIbMaxIters);
+  PC_TRY(pc::wait_status(p));
   if (cudaSetDevice(p->device) != cudaSuccess) return pc::fail(PC_ERR_CUDA, "cannot select device %d", p->device);
   if (!pc::is_device_ptr(u_star) || (f_ib_init && !pc::is_device_ptr(f_ib_init)) || !pc::is_device_ptr(p_out) ||
       !pc::is_device_ptr(u_out) || (f_ib_out && !pc::is_device_ptr(f_ib_out)))

@@ -258,7 +258,7 @@ __global__ void __launch_bounds__(kResidentThreads, 1) resident_kernel(const __g
       }
       if (j == R.sweeps && final_pass) break;
       if constexpr (CLUSTER) cluster_barrier();
-      else good = grid_barrier(R.bar, phase, R.st);
+      else good = grid_barrier(R.bar, phase, R.polls);
       if (first && j > 0 && R.adaptive && good) {
         if (threadIdx.x == 0) stop = refine_stopped_before(R.st, j, R.tol) ? 1 : 0;
         __syncthreads();
@@ -283,14 +283,14 @@ __global__ void __launch_bounds__(kResidentThreads, 1) resident_kernel(const __g
       f[1] = make_double2(f2d_bits(h[2]) + f2d_bits(l[2]), f2d_bits(h[3]) + f2d_bits(l[3]));
     }
   }
-  if (!CLUSTER && threadIdx.x == 0) {
-    if (!good) {   // a barrier gave up: the result is not one
-      R.f64[0] = __longlong_as_double(0x7ff8000000000000LL);
-      R.p2[0] = make_float2(__int_as_float(0x7fc00000), 0.0f);
-    } else if (atomicAdd(R.bar + 1, 1u) == gridDim.x - 1) {   // the last CTA leaves the counters at zero
-      R.bar[0] = 0u;
-      R.bar[1] = 0u;
-    }
+  if constexpr (!CLUSTER) {
+    if (!good)   // a barrier gave up: these rows have no result
+      for (int i = threadIdx.x; i < o.lines * nl; i += blockDim.x) {
+        R.p2[o.line0 * nl + i] = make_float2(__int_as_float(0x7fc00000), 0.0f);
+        R.f64[o.line0 * nl + i] = __longlong_as_double(0x7ff8000000000000LL);
+      }
+    __syncthreads();
+    if (threadIdx.x == 0) leave_grid(R.bar, good, R.gave_up);
   }
 }
 

@@ -23,6 +23,8 @@ struct ResidentArgs {
   int row_tiles;             // row tiles per CTA (consecutive)
   int own_at;                // slots of shared memory before the own rows' planes
   float tol;
+  unsigned polls;            // of one grid barrier at most
+  unsigned *gave_up;         // host word: set where a barrier ran out of them
 };
 
 // The plain FP64 solve of a small grid: its passes, the gauge and p in one launch (resident64.cu).
@@ -36,6 +38,8 @@ struct Resident64Args {
   int grid, cluster, row_tiles, tables_at, own_at;
   int gauge;                 // 0 none, 1 zero mean, 2 zero first cell
   double inv_cells;
+  unsigned polls;
+  unsigned *gave_up;
 };
 pc_status launch_resident64(const Resident64Args &R, int dim, size_t smem, cudaStream_t st);
 pc_status prepare_resident64();
@@ -47,9 +51,10 @@ int resident_cluster_size();
 
 #ifdef __CUDACC__
 // Barrier of the whole grid (a cooperative launch: every CTA is resident). bar counts arrivals;
-// phase is the number of barriers passed. Bounded: after about two seconds it gives up, marks the
-// statistics and returns false (every CTA that waits does), and the caller leaves the kernel.
-__device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned &phase, DevStats *st) {
+// phase is the number of barriers passed. Bounded: after `polls` looks at the count it gives up and
+// returns false, and the caller leaves the kernel. A CTA that left does not arrive at the next barrier,
+// so every other CTA gives up there at the latest.
+__device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned &phase, unsigned polls) {
   __shared__ int ok;
   __syncthreads();
   ++phase;
@@ -58,18 +63,29 @@ __device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned &phase, Dev
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
     unsigned seen = 0;
     int good = 0;
-    for (int it = 0; it < (1 << 22); ++it) {
+    for (unsigned it = 0; it < polls; ++it) {
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
       if (seen >= want) {
         good = 1;
         break;
       }
     }
-    if (!good) atomicOr(&st->flags, (unsigned)FLAG_TIMEOUT);
     ok = good;
   }
   __syncthreads();
   return ok != 0;
+}
+// End of a kernel with grid barriers, by one thread of each CTA: the host learns of a barrier that gave up
+// (its CTA has filled its rows of the result with NaN), and the last CTA leaves the counters at zero.
+__device__ __forceinline__ void leave_grid(unsigned *bar, bool good, unsigned *gave_up) {
+  if (!good) {
+    *reinterpret_cast<volatile unsigned *>(gave_up) = 1u;
+    __threadfence_system();
+  }
+  if (atomicAdd(bar + 1, 1u) == gridDim.x - 1) {
+    bar[0] = 0u;
+    bar[1] = 0u;
+  }
 }
 
 // Barrier of a grid that is one cluster: the hardware's (0.2 us against 1.2 for the grid barrier).

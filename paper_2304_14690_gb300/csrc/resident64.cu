@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(kResidentThreads, 1) resident64_kernel(const _
     }
     if (final_pass) break;
     if constexpr (CLUSTER) cluster_barrier();
-    else good = grid_barrier(R.bar, phase, R.st);
+    else good = grid_barrier(R.bar, phase, R.polls);
   }
   __syncthreads();
   const int cells = lines * nl, c0 = line0 * nl;
@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(kResidentThreads, 1) resident64_kernel(const _
       if (c0 == 0 && cells > 0) R.st->corner_p = own[0];
     }
     if constexpr (CLUSTER) cluster_barrier();
-    else good = grid_barrier(R.bar, phase, R.st);
+    else good = grid_barrier(R.bar, phase, R.polls);
     double t = 0.0;
     for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) t += __ldcg(R.partials + b);
     t = cta_sum(t);
@@ -119,13 +119,11 @@ __global__ void __launch_bounds__(kResidentThreads, 1) resident64_kernel(const _
       const double2 v = *reinterpret_cast<const double2 *>(own + i);
       *reinterpret_cast<double2 *>(R.p + c0 + i) = make_double2(v.x - shift, v.y - shift);
     }
-  if (!CLUSTER && threadIdx.x == 0) {
-    if (!good) {   // a barrier gave up: the result is not one
-      R.p[0] = __longlong_as_double(0x7ff8000000000000LL);
-    } else if (atomicAdd(R.bar + 1, 1u) == gridDim.x - 1) {   // the last CTA leaves the counters at zero
-      R.bar[0] = 0u;
-      R.bar[1] = 0u;
-    }
+  if constexpr (!CLUSTER) {
+    if (!good)   // a barrier gave up: these rows have no result
+      for (int i = threadIdx.x; i < cells; i += blockDim.x) R.p[c0 + i] = __longlong_as_double(0x7ff8000000000000LL);
+    __syncthreads();
+    if (threadIdx.x == 0) leave_grid(R.bar, good, R.gave_up);
   }
 }
 

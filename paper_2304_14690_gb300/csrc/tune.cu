@@ -131,7 +131,7 @@ static pc_status autotune(Plan *p, cudaStream_t st, double *best_out) {
   cudaEventDestroy(e1);
   plan_drop_graphs(p);
   if (best_out) *best_out = best;
-  return status;
+  return status == PC_OK ? wait_status(p) : status;
 }
 
 }  // namespace pc

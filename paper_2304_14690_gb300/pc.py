@@ -163,6 +163,7 @@ FUNCTIONS = {
                                            ctypes.c_void_p, ctypes.c_void_p]),
     "pc_momentum_reset": (ctypes.c_int, [ctypes.c_void_p]),
     "pc_momentum_destroy": (ctypes.c_int, [ctypes.c_void_p]),
+    "pc_plan_set_wait_limit": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_uint]),
     "pc_status_string": (ctypes.c_char_p, [ctypes.c_int]),
     "pc_last_error_message": (ctypes.c_char_p, []),
 }
@@ -334,6 +335,10 @@ class Plan:
         b = ctypes.c_size_t()
         _check(load().pc_plan_bytes(self.handle, ctypes.byref(b)))
         return b.value
+
+    def set_wait_limit(self, polls):
+        """Polls of one wait inside a one-launch solve at most; 0: one launch per pass and no waits."""
+        _check(load().pc_plan_set_wait_limit(self.handle, polls))
 
     def graphs(self, on=True):
         _check(load().pc_set_graphs(self.handle, 1 if on else 0))
