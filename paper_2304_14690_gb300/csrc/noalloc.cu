@@ -22,7 +22,6 @@ constexpr long long kStaticMaxCells = 1LL << 19;
 constexpr long long kStaticDoubles = 1LL << 20;   // 8 MiB
 static __device__ __align__(256) double g_static_scratch[kStaticDoubles];
 
-constexpr int kMaxDevices = 64;
 static void *g_static_ptr[kMaxDevices] = {nullptr};
 static std::mutex g_static_mutex;
 

@@ -11,6 +11,7 @@
 //
 // Mixed precision: the transforms run in FP32; the iterate p is kept in FP64 and corrected by
 // sweeps p += solve32(s - L_h p) whose residual is formed in FP64 (iterative refinement).
+#include <atomic>
 #include <cmath>
 #include <cstdint>
 #include <cstdio>
@@ -258,6 +259,18 @@ static bool quad_io(const Plan *p, const PassSpec &ps, bool fp32) {
          (!row || (aligned16(ps.src) && aligned16(ps.dst) && aligned16(ps.f64)));
 }
 
+// SMs of a device (of the part of it that the process may use), asked for once.
+static int sm_count(int device) {
+  static std::atomic<int> known[kMaxDevices];
+  if (device < 0 || device >= kMaxDevices) return 1;
+  int n = known[device].load(std::memory_order_relaxed);
+  if (n == 0) {
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || n < 1) n = 1;
+    known[device].store(n, std::memory_order_relaxed);
+  }
+  return n;
+}
+
 template <typename Real>
 pc_status build_pass(const Plan *p, const PassSpec &ps, PassArgs<Real> &A, long long &tiles, int &threads,
                      size_t &smem, int batch_threads) {
@@ -293,9 +306,9 @@ pc_status build_pass(const Plan *p, const PassSpec &ps, PassArgs<Real> &A, long 
     int L = axis == p->dim - 1 ? 1 : 4;   // column tiles: four lines fill half a sector in FP32, one in FP64
     while (L < 32 && 2 * L * M <= slots) L *= 2;
     if (batch_threads <= 0) {
-      const long long lines = p->ncells / ax.n;
-      while (L > 4 && lines / L < 2 * 152) L /= 2;
-      while (L > 1 && lines / L < 152) L /= 2;   // few long lines (1024 x 96 in FP64: 152 us at four lines, 57 at one)
+      const long long lines = p->ncells / ax.n, sms = sm_count(p->device);
+      while (L > 4 && lines / L < 2 * sms) L /= 2;
+      while (L > 1 && lines / L < sms) L /= 2;   // few long lines (1024 x 96 in FP64: 152 us at four lines, 57 at one)
     }
     while (L > 1 && loop::tile_smem<Real>(M, L) > 160 * 1024) L /= 2;
     tiles = fill_loop<Real>(p, ps, A, L);
@@ -475,7 +488,7 @@ static void tables_of(const AxisInfo &ax, int &first, int &end) {
 // all SMs, 160 x 200 62 against 52; 3D: 20^3 80 against 84, 24^3 74 against 72).
 constexpr long long kClusterCells2D = 20000, kClusterCells3D = 8192;
 static bool cluster_grid(const Plan *p) {
-  return p->ncells <= (p->dim == 2 ? kClusterCells2D : kClusterCells3D) && resident_cluster_size() > 0;
+  return p->ncells <= (p->dim == 2 ? kClusterCells2D : kClusterCells3D) && resident_cluster_size(p->device) > 0;
 }
 
 // Tiles, tables and own rows of a cooperative solve's passes: lines per tile as few as give every SM
@@ -534,14 +547,17 @@ static bool resident_layout(const Plan *p, const std::vector<PassSpec> &specs, P
   return fits;
 }
 
-static int sm_count() {
-  static const int sms = [] {
-    int dev = 0, n = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    return n;
-  }();
-  return sms;
+// A grid that does not fit at once (a context held to fewer SMs than the device reports) is not launched:
+// the solve takes one launch per pass.
+static pc_status resident_taken(Plan *p, cudaError_t e, bool &taken) {
+  if (e == cudaErrorCooperativeLaunchTooLarge) {
+    cudaGetLastError();
+    return PC_OK;
+  }
+  PC_CUDA_TRY(e);
+  count_launch(p);
+  taken = true;
+  return PC_OK;
 }
 
 pc_status solve_resident(Plan *p, const double *s64, const float2 *s2, double *pout, int sweeps, bool adaptive,
@@ -559,7 +575,7 @@ pc_status solve_resident(Plan *p, const double *s64, const float2 *s2, double *p
   R.cluster = cluster_grid(p);
   size_t smem = 0;
   if (!resident_layout<float>(p, solve_pass_specs(p, true, SRC_F32, rs, DST_PAIR_SET, p->p2), R.pass,
-                              R.cluster ? resident_cluster_size() : sm_count(), 2 * kLoopSlots, 16, R.grid, R.row_tiles,
+                              R.cluster ? resident_cluster_size(p->device) : sm_count(p->device), 2 * kLoopSlots, 16, R.grid, R.row_tiles,
                               R.tables_at, R.own_at, smem))
     return PC_OK;
   R.g = g;
@@ -574,10 +590,7 @@ pc_status solve_resident(Plan *p, const double *s64, const float2 *s2, double *p
   R.tol = tol;
   R.polls = p->wait_polls;
   R.gave_up = p->gave_up;
-  PC_TRY(launch_resident(R, p->dim, s2 != nullptr, smem, st));
-  count_launch(p);
-  taken = true;
-  return PC_OK;
+  return resident_taken(p, launch_resident(R, p->dim, s2 != nullptr, smem, st), taken);
 }
 
 // Largest grid of the FP64 solve in one launch (96^3 236 us against 275 by launches, 512^2 76 against
@@ -592,10 +605,10 @@ pc_status solve_resident64(Plan *p, const double *s, double *pout, int gauge, cu
     if (p->ax[a].slots64 != 2 || p->ax[a].loop_nst == 0 || p->ax[a].M > 1024) return PC_OK;
   Resident64Args R;
   memset(&R, 0, sizeof(R));
-  R.cluster = p->ncells <= kCluster64Cells && resident_cluster_size() > 0;
+  R.cluster = p->ncells <= kCluster64Cells && resident_cluster_size(p->device) > 0;
   size_t smem = 0;
   if (!resident_layout<double>(p, solve_pass_specs(p, false, SRC_F64, s, DST_F64_SET, pout), R.pass,
-                               R.cluster ? resident_cluster_size() : sm_count(), kLoopSlots, 8, R.grid, R.row_tiles,
+                               R.cluster ? resident_cluster_size(p->device) : sm_count(p->device), kLoopSlots, 8, R.grid, R.row_tiles,
                                R.tables_at, R.own_at, smem))
     return PC_OK;
   if (R.grid > 2 * (p->ncells / 256) + 64) return PC_OK;   // the partial sums' array (partial_slots)
@@ -608,10 +621,7 @@ pc_status solve_resident64(Plan *p, const double *s, double *pout, int gauge, cu
   R.inv_cells = 1.0 / (double)p->ncells;
   R.polls = p->wait_polls;
   R.gave_up = p->gave_up;
-  PC_TRY(launch_resident64(R, p->dim, smem, st));
-  count_launch(p);
-  taken = true;
-  return PC_OK;
+  return resident_taken(p, launch_resident64(R, p->dim, smem, st), taken);
 }
 
 pc_status solve_fp64_grid(Plan *p, const double *s, double *pout, cudaStream_t st) {

@@ -18,6 +18,7 @@
 // 261 -> 199. A phase of the 1024 x 512 grid takes about 7 us: five half-stages per transform at
 // 0.35 us each (latency and issue alike: 38% of the issue slots), 1 us to load, 1 to store, the
 // barrier.
+#include <atomic>
 #include <type_traits>
 
 #include "loop_pass.cuh"
@@ -295,7 +296,7 @@ __global__ void __launch_bounds__(kResidentThreads, 1) resident_kernel(const __g
 }
 
 template <int DIM, typename SV, bool IEEE>
-static pc_status launch(const ResidentArgs &R, size_t smem, cudaStream_t st) {
+static cudaError_t launch(const ResidentArgs &R, size_t smem, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)R.grid);
   cfg.blockDim = dim3(kResidentThreads);
@@ -311,17 +312,16 @@ static pc_status launch(const ResidentArgs &R, size_t smem, cudaStream_t st) {
     at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.numAttrs = tl_plain_launch ? 1 : 2;
-    PC_CUDA_TRY(cudaLaunchKernelEx(&cfg, resident_kernel<DIM, SV, true, IEEE>, R));
+    return cudaLaunchKernelEx(&cfg, resident_kernel<DIM, SV, true, IEEE>, R);
   } else {
     at[0].id = cudaLaunchAttributeCooperative;
     at[0].val.cooperative = 1;
     cfg.numAttrs = 1;
-    PC_CUDA_TRY(cudaLaunchKernelEx(&cfg, resident_kernel<DIM, SV, false, IEEE>, R));
+    return cudaLaunchKernelEx(&cfg, resident_kernel<DIM, SV, false, IEEE>, R);
   }
-  return PC_OK;
 }
 
-pc_status launch_resident(const ResidentArgs &R, int dim, bool pairs, size_t smem, cudaStream_t st) {
+cudaError_t launch_resident(const ResidentArgs &R, int dim, bool pairs, size_t smem, cudaStream_t st) {
   auto of = [&](auto ieee) {
     constexpr bool I = decltype(ieee)::value;
     if (dim == 2) return pairs ? launch<2, float2, I>(R, smem, st) : launch<2, double, I>(R, smem, st);
@@ -348,26 +348,32 @@ pc_status prepare_resident() {
   return prepare_one<3, double, true>();
 }
 
-int resident_cluster_size() {
-  static const int size = [] {
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
-    cfg.blockDim = dim3(kResidentThreads);
-    cfg.dynamicSmemBytes = kResidentSmem;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    for (int n : {16, 8}) {
-      at[0].val.clusterDim.x = (unsigned)n;
-      cfg.gridDim = dim3((unsigned)n);
-      int fit = 0;
-      if (cudaOccupancyMaxActiveClusters(&fit, resident_kernel<3, double, true, true>, &cfg) == cudaSuccess && fit > 0) return n;
-      cudaGetLastError();
+int resident_cluster_size(int device) {
+  static std::atomic<int> known[kMaxDevices];   // 1 + the size
+  if (device < 0 || device >= kMaxDevices) return 0;
+  const int have = known[device].load(std::memory_order_relaxed);
+  if (have) return have - 1;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  cfg.blockDim = dim3(kResidentThreads);
+  cfg.dynamicSmemBytes = kResidentSmem;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  int size = 0;
+  for (int n : {16, 8}) {
+    at[0].val.clusterDim.x = (unsigned)n;
+    cfg.gridDim = dim3((unsigned)n);
+    int fit = 0;
+    if (cudaOccupancyMaxActiveClusters(&fit, resident_kernel<3, double, true, true>, &cfg) == cudaSuccess && fit > 0) {
+      size = n;
+      break;
     }
-    return 0;
-  }();
+    cudaGetLastError();
+  }
+  known[device].store(1 + size, std::memory_order_relaxed);
   return size;
 }
 

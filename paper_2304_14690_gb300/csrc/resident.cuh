@@ -41,13 +41,13 @@ struct Resident64Args {
   unsigned polls;
   unsigned *gave_up;
 };
-pc_status launch_resident64(const Resident64Args &R, int dim, size_t smem, cudaStream_t st);
+cudaError_t launch_resident64(const Resident64Args &R, int dim, size_t smem, cudaStream_t st);
 pc_status prepare_resident64();
 
-pc_status launch_resident(const ResidentArgs &R, int dim, bool pairs, size_t smem, cudaStream_t st);
+cudaError_t launch_resident(const ResidentArgs &R, int dim, bool pairs, size_t smem, cudaStream_t st);
 pc_status prepare_resident();
-// CTAs of the largest cluster the kernel runs as (16, else 8; 0: none).
-int resident_cluster_size();
+// CTAs of the largest cluster the kernel runs as on the device, which is current (16, else 8; 0: none).
+int resident_cluster_size(int device);
 
 #ifdef __CUDACC__
 // Barrier of the whole grid (a cooperative launch: every CTA is resident). bar counts arrivals;

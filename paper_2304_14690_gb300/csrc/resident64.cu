@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(kResidentThreads, 1) resident64_kernel(const _
 }
 
 template <int DIM>
-static pc_status launch64(const Resident64Args &R, size_t smem, cudaStream_t st) {
+static cudaError_t launch64(const Resident64Args &R, size_t smem, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)R.grid);
   cfg.blockDim = dim3(kResidentThreads);
@@ -144,17 +144,16 @@ static pc_status launch64(const Resident64Args &R, size_t smem, cudaStream_t st)
     at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.numAttrs = tl_plain_launch ? 1 : 2;
-    PC_CUDA_TRY(cudaLaunchKernelEx(&cfg, resident64_kernel<DIM, true>, R));
+    return cudaLaunchKernelEx(&cfg, resident64_kernel<DIM, true>, R);
   } else {
     at[0].id = cudaLaunchAttributeCooperative;
     at[0].val.cooperative = 1;
     cfg.numAttrs = 1;
-    PC_CUDA_TRY(cudaLaunchKernelEx(&cfg, resident64_kernel<DIM, false>, R));
+    return cudaLaunchKernelEx(&cfg, resident64_kernel<DIM, false>, R);
   }
-  return PC_OK;
 }
 
-pc_status launch_resident64(const Resident64Args &R, int dim, size_t smem, cudaStream_t st) {
+cudaError_t launch_resident64(const Resident64Args &R, int dim, size_t smem, cudaStream_t st) {
   return dim == 2 ? launch64<2>(R, smem, st) : launch64<3>(R, smem, st);
 }
 
