@@ -11,6 +11,7 @@
 //
 // Mixed precision: the transforms run in FP32; the iterate p is kept in FP64 and corrected by
 // sweeps p += solve32(s - L_h p) whose residual is formed in FP64 (iterative refinement).
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstdint>
@@ -491,13 +492,20 @@ static bool cluster_grid(const Plan *p) {
   return p->ncells <= (p->dim == 2 ? kClusterCells2D : kClusterCells3D) && resident_cluster_size(p->device) > 0;
 }
 
+// Slots up to which a tile of the cooperative solve takes more lines where more CTAs would not be faster
+// (FP64: half of them): the grid leaves SMs to solves on other streams. Projections in us, one after the
+// other / on 8 streams: 256^2 mixed 64 CTAs 75.9 / 26.4, 128 CTAs 75.5 / 48.7, 32 CTAs 78.6 / 15.7; 192^2
+// 48 CTAs 69.4 / 18.8, 96 CTAs 68.0 / 49.9, 24 CTAs 75.3 / 11.4; 32^3 32 CTAs 115.5 / 21.8, 128 CTAs 113.7 /
+// 66.1; FP64 128^2 32 CTAs 54.4 / 10.2, 128 CTAs 54.3 / 35.1; 256^2 64 CTAs 70.9 / 25.4, 128 CTAs 65.8 / 40.7.
+constexpr int kSpreadSlots = 512;
+
 // Tiles, tables and own rows of a cooperative solve's passes: lines per tile as few as give every SM
-// at most one tile, and fewer again where the buffers would not leave room for the own rows
+// at most one tile, more while the tile has no more than `spread` slots, and fewer again where the buffers would not leave room for the own rows
 // (own_bytes per cell). Behind the tiles: per axis the wrappers' factors its family reads, the stage
 // twiddles and, on the dividing pass, the eigenvalues.
 template <typename Real>
-static bool resident_layout(const Plan *p, const std::vector<PassSpec> &specs, PassArgs<Real> *pass, int sms, int cap0,
-                            int own_bytes, int &grid, int &row_tiles, int &tables_at, int &own_at, size_t &smem) {
+static bool resident_layout(const Plan *p, const std::vector<PassSpec> &specs, PassArgs<Real> *pass, int sms, int spread,
+                            int cap0, int own_bytes, int &grid, int &row_tiles, int &tables_at, int &own_at, size_t &smem) {
   constexpr int kSlot = 2 * (int)sizeof(Real);
   const int np = (int)specs.size(), last = p->dim - 1;
   int slots = 0, at[3][3];
@@ -522,6 +530,7 @@ static bool resident_layout(const Plan *p, const std::vector<PassSpec> &specs, P
       const long long lines = p->ncells / p->ax[specs[k].axis].n;
       int L = 1;
       while ((lines + L - 1) / L > sms && 2 * L * M <= cap) L *= 2;
+      while (2 * L * M <= spread) L *= 2;
       const long long tiles = fill_loop<Real>(p, specs[k], pass[k], L);
       most = tiles > most ? tiles : most;
       const size_t b = loop::tile_smem<Real>(M, L);
@@ -575,7 +584,8 @@ pc_status solve_resident(Plan *p, const double *s64, const float2 *s2, double *p
   R.cluster = cluster_grid(p);
   size_t smem = 0;
   if (!resident_layout<float>(p, solve_pass_specs(p, true, SRC_F32, rs, DST_PAIR_SET, p->p2), R.pass,
-                              R.cluster ? resident_cluster_size(p->device) : sm_count(p->device), 2 * kLoopSlots, 16, R.grid, R.row_tiles,
+                              R.cluster ? resident_cluster_size(p->device) : sm_count(p->device),
+                              R.cluster ? 0 : kSpreadSlots, 2 * kLoopSlots, 16, R.grid, R.row_tiles,
                               R.tables_at, R.own_at, smem))
     return PC_OK;
   R.g = g;
@@ -608,7 +618,8 @@ pc_status solve_resident64(Plan *p, const double *s, double *pout, int gauge, cu
   R.cluster = p->ncells <= kCluster64Cells && resident_cluster_size(p->device) > 0;
   size_t smem = 0;
   if (!resident_layout<double>(p, solve_pass_specs(p, false, SRC_F64, s, DST_F64_SET, pout), R.pass,
-                               R.cluster ? resident_cluster_size(p->device) : sm_count(p->device), kLoopSlots, 8, R.grid, R.row_tiles,
+                               R.cluster ? resident_cluster_size(p->device) : sm_count(p->device),
+                               R.cluster ? 0 : kSpreadSlots / 2, kLoopSlots, 8, R.grid, R.row_tiles,
                                R.tables_at, R.own_at, smem))
     return PC_OK;
   if (R.grid > 2 * (p->ncells / 256) + 64) return PC_OK;   // the partial sums' array (partial_slots)
