@@ -163,9 +163,8 @@ __device__ __forceinline__ void stage16_split(typename Cplx<Real>::T *in, typena
 }
 
 // Forward FFT of every line of the tile, ping-ponging between a and b; the result is left in a.
-// Called by every thread of the CTA, after a barrier; ends with one. SPLIT: radix-16 stages as
-// their halves.
-template <typename Real, bool SPLIT, typename Tables>
+// Called by every thread of the CTA, after a barrier; ends with one. Radix-16 stages run as their halves.
+template <typename Real, typename Tables>
 __device__ __forceinline__ void fft(const PassArgs<Real> &A, int L, int LS, typename Cplx<Real>::T *&a,
                                     typename Cplx<Real>::T *&b, const Tables &tb, int pre,
                                     const typename Cplx<Real>::T *w16tab) {
@@ -175,7 +174,7 @@ __device__ __forceinline__ void fft(const PassArgs<Real> &A, int L, int LS, type
   for (int s = 0; s < nst; ++s) {
     const StageInfo si = A.st[s];
     const int p0 = s == 0 ? pre : -1;
-    if (SPLIT && si.R == 16) {
+    if (si.R == 16) {
       stage16_split<Real>(a, b, L, LS, si, tb, p0, w16tab);
       __syncthreads();
       continue;
@@ -184,9 +183,7 @@ __device__ __forceinline__ void fft(const PassArgs<Real> &A, int L, int LS, type
     // end their loops at different iterations into the barrier in parts (a 60 x 720 solve off by 5e4,
     // differently in each run). The warp barrier below is there for the same reason.
     const int radix = si.R;
-    if (radix == 16) {
-      if constexpr (!SPLIT) stage<Real, 16>(a, b, L, LS, si, tb, p0);
-    } else if (radix == 8) stage<Real, 8>(a, b, L, LS, si, tb, p0);
+    if (radix == 8) stage<Real, 8>(a, b, L, LS, si, tb, p0);
     else if (radix == 4) stage<Real, 4>(a, b, L, LS, si, tb, p0);
     else if (radix == 2) stage<Real, 2>(a, b, L, LS, si, tb, p0);
     else if (radix == 3) stage<Real, 3>(a, b, L, LS, si, tb, p0);
@@ -518,9 +515,10 @@ __device__ __forceinline__ void load_coefs(const PassArgs<Real> &A, const Tile &
 
 // One pass over a tile: [forward transform] [division] [inverse transform] as A asks. quad(l, base,
 // qd, stride) yields the input values at positions 4 qd .. 4 qd + 3 of line l (first cell base), and
-// put(l, base, qd, stride, x) takes the outputs of a final inverse. buf: two buffers of L lines, then the lines' eigenvalue sums. The two halves share one copy
-// of the FFT (a loop that is not unrolled). The caller puts a barrier before it; it ends without.
-template <typename Real, bool SPLIT, bool IEEE, typename Tables, typename QuadFn, typename PutFn>
+// put(l, base, qd, stride, x) takes the outputs of a final inverse. buf: two buffers of L lines, then the
+// lines' eigenvalue sums. The two halves share one copy of the FFT (a loop that is not unrolled). The
+// caller puts a barrier before it; it ends without.
+template <typename Real, bool IEEE, typename Tables, typename QuadFn, typename PutFn>
 __device__ __forceinline__ void pass_tile(const PassArgs<Real> &A, int tile, typename Cplx<Real>::T *buf,
                                           const Tables &tb, const typename Cplx<Real>::T *w16tab, QuadFn quad, PutFn put) {
   using T = typename Cplx<Real>::T;
@@ -547,7 +545,7 @@ __device__ __forceinline__ void pass_tile(const PassArgs<Real> &A, int tile, typ
   __syncthreads();
 #pragma unroll 1
   for (int half = fwd ? 0 : 1; half < (inv ? 2 : 1); ++half) {
-    fft<Real, SPLIT>(A, t.L, t.LS, a, b, tb, fam == 2 && half == 0 ? tw_dct4pre(M) : -1, w16tab);
+    fft<Real>(A, t.L, t.LS, a, b, tb, fam == 2 && half == 0 ? tw_dct4pre(M) : -1, w16tab);
     if (half == 0 && inv) {
       if (fam == 0) divide_tile<Real, 0, IEEE>(A, t, a, lam, tb);
       else if (fam == 1) divide_tile<Real, 1, IEEE>(A, t, a, lam, tb);
@@ -578,14 +576,14 @@ __device__ __forceinline__ void pass_tile(const PassArgs<Real> &A, int tile, typ
 }
 
 // The pass on its plain source.
-template <typename Real, bool SPLIT, bool IEEE>
+template <typename Real, bool IEEE>
 __device__ __forceinline__ void pass_tile(const PassArgs<Real> &A, int tile, typename Cplx<Real>::T *buf,
                                           const typename Cplx<Real>::T *w16tab) {
   const void *src = A.src;
   const int mode = A.src_mode;
   const GlobalTables<Real> tb{A.tw, A.stw, A.lam[A.axis]};
   const Store<Real> out = store_of(A);
-  pass_tile<Real, SPLIT, IEEE>(
+  pass_tile<Real, IEEE>(
       A, tile, buf, tb, w16tab,
       [&](int, int base, int qd, int stride) { return load_src4<Real>(src, mode, base + 4 * qd * stride, stride); },
       [&](int, int base, int qd, int stride, const Quad<Real> &x) { store_dst4(out, base + 4 * qd * stride, stride, x); });

@@ -391,10 +391,11 @@ pc_status solve_fp32_grid(Plan *p, int src_mode, const void *s, int dst_mode, vo
 constexpr long long kResidentCells = 1LL << 20;
 // Geometry of a plan's pressure grid for the cell kernels (project.cu).
 GridDev grid_dev(const Plan *p);
+// A solve with a fixed number of sweeps and no gauge, as the autotuner times it.
+pc_status solve_fixed_sweeps(Plan *p, const double *s64, double *pout, int sweeps, cudaStream_t st);
 // The refined FP32 solve as one cooperative kernel (resident.cu) where the plan and the arrays allow
 // it; taken says whether it was launched. s2 (nullable): the source as (hi, lo) pairs, else FP64 in
 // s64. The iterate is left in p->p2 and, in FP64, in pout.
-pc_status solve_fixed_sweeps(Plan *p, const double *s64, double *pout, int sweeps, cudaStream_t st);
 pc_status solve_resident(Plan *p, const double *s64, const float2 *s2, double *pout, int sweeps, bool adaptive,
                          float tol, const GridDev &g, cudaStream_t st, bool &taken);
 // The plain FP64 solve of a small grid with its gauge (gauge_mode) as one launch (resident64.cu).
@@ -406,8 +407,8 @@ void plan_drop_graphs(Plan *p);
 // ----------------------------------------------------------------------------- batches
 // Stages of the batched pipeline (one launch per stage for all problems of a batch).
 enum BatchStage {
-  BATCH_PREP = 1, BATCH_TRANSFER = 2 /* +axis */, BATCH_DIVERGENCE = 5, BATCH_RESIDUAL = 6,
-  BATCH_GAUGE_SUM = 7, BATCH_FINALIZE = 8, BATCH_GRADIENT = 9, BATCH_STAGES = 10
+  BATCH_PREP = 0, BATCH_TRANSFER = 1 /* +axis */, BATCH_DIVERGENCE = 4, BATCH_RESIDUAL = 5,
+  BATCH_GAUGE_SUM = 6, BATCH_FINALIZE = 7, BATCH_GRADIENT = 8, BATCH_STAGES = 9
 };
 
 // Per-problem parameters of a batched launch (device array, one entry per problem).

@@ -2,15 +2,15 @@
 //   1. forward 1D transforms along each axis in turn,
 //   2. division by the sum of the 1D eigenvalues of the central-difference Laplacian,
 //   3. backward 1D transforms.
-// One kernel launch per axis pass; grids up to about a million cells take all the passes of an FP32
-// refined solve in one cooperative launch (resident.cu). The contiguous (last) axis is processed in row tiles, the
-// other axes in column tiles of W adjacent lines so that every global access is coalesced
-// without a transpose. The division is fused into the pass of axis 0, which does its forward
+// One kernel launch per axis pass; grids up to about a million cells take all the passes of a solve in
+// one launch (resident.cu, resident64.cu). The contiguous (last) axis is processed in row tiles, the
+// other axes in column tiles of adjacent lines so that every global access is coalesced without a
+// transpose. The division is fused into the pass of axis 0, which does its forward
 // transform, the division and its inverse transform on the tile while it sits in shared memory.
 // 2D: [fwd ax1] -> [fwd ax0, divide, inv ax0] -> [inv ax1]; 3D adds ax1 passes around the middle.
 //
-// Mixed precision: the transforms run in FP32; the iterate p is kept in FP64 and corrected by
-// sweeps p += solve32(s - L_h p) whose residual is formed in FP64 (iterative refinement).
+// Mixed precision: the transforms run in FP32; the iterate p is kept as FP32 (hi, lo) pairs and corrected
+// by sweeps p += solve32(s - L_h p) whose residual is formed on such pairs (iterative refinement).
 #include <algorithm>
 #include <atomic>
 #include <cmath>
@@ -500,8 +500,8 @@ static bool cluster_grid(const Plan *p) {
 constexpr int kSpreadSlots = 512;
 
 // Tiles, tables and own rows of a cooperative solve's passes: lines per tile as few as give every SM
-// at most one tile, more while the tile has no more than `spread` slots, and fewer again where the buffers would not leave room for the own rows
-// (own_bytes per cell). Behind the tiles: per axis the wrappers' factors its family reads, the stage
+// at most one tile, more while the tile has no more than `spread` slots, and fewer again where the
+// buffers would not leave room for the own rows (own_bytes per cell). Behind the tiles: per axis the wrappers' factors its family reads, the stage
 // twiddles and, on the dividing pass, the eigenvalues.
 template <typename Real>
 static bool resident_layout(const Plan *p, const std::vector<PassSpec> &specs, PassArgs<Real> *pass, int sms, int spread,

@@ -235,9 +235,11 @@ __global__ void transfer64_kernel(int rows, int K, const int32_t *__restrict__ c
 
 // KC > 0: the neighbour count is a compile-time constant and the loop is unrolled, so all
 // index and weight loads are in flight before the dependent gathers (memory-level parallelism).
-// The gathers' registers are bounded for the number of warps that keeps most bytes in flight: 32
-// (2D: eight CTAs of 256 threads per SM) and 48 registers (3D transfers: five; unbounded the
-// compiler takes 53 to 124), 32 and 40 for the gradients. 256x128x128 box: 1857 -> 1639 us.
+// The gathers' registers are bounded for the number of warps that keeps most bytes in flight: 32 (eight
+// CTAs of 256 threads per SM) for 2D transfers, 2D gradients and the single 3D gradient of the mixed
+// path, 48 (five CTAs) for 3D transfers (unbounded the compiler takes 53 to 124), 40 (six) for the FP64 and
+// the batched 3D gradients. 256x128x128 box: 1857 -> 1639 us. At 32 registers the 3D mixed gradient spills
+// 28 bytes per thread (68 read back, in L1); with 40 and six CTAs the box takes 1641.
 // The gathered node value as an FP32 (hi, lo) pair, here the pairs of u~ that prep wrote. F64: the
 // plan's solve is not refined, so the last bit of the source's FP32 copy shows in the result (4.8e-8
 // of p over 24 problems), and the fluxes take the rounding to FP64 that they always had there. A
@@ -977,7 +979,7 @@ __device__ __forceinline__ void gradient_mixed_kernel_body(const VBlock &vb, int
   }
 }
 template <typename VT, int DIM>
-__global__ void __launch_bounds__(256, DIM == 2 ? 8 : 8) gradient_mixed_kernel(int N, BlockGrid bg, const int32_t *__restrict__ col,
+__global__ void __launch_bounds__(256, 8) gradient_mixed_kernel(int N, BlockGrid bg, const int32_t *__restrict__ col,
                                       const float2 *__restrict__ D2, const float2 *__restrict__ p2,
                                       const uint8_t *__restrict__ type, const VT *__restrict__ u,
                                       double inv_dt, double dt, double beta, VT *__restrict__ uo,
@@ -1322,6 +1324,8 @@ __global__ void batch_divergence(const BatchProblem *__restrict__ P, const int *
 // do not depend on how blocks are grouped), so a skipped
 // launch costs a quarter of the CTAs.
 constexpr int kResidualChunk = 4;
+// 64 registers (four CTAs per SM); in 3D 100 bytes per thread spill (three CTAs without: 12 requests of the
+// stream 1428 us against 1461).
 template <int DIM>
 __global__ void __launch_bounds__(256, 4) batch_residual(const BatchProblem *__restrict__ P, const int *__restrict__ seg, int count, int k) {
   pdl_enter();
@@ -1411,7 +1415,6 @@ void batch_launch(int stage, int variant, const BatchProblem *P, const int *seg,
 void batch_block_counts(const Plan *p, int *nb) {
   const long long N = p->N, nc = p->ncells;
   const GridDev g = grid_dev(p);
-  nb[0] = 0;
   nb[BATCH_PREP] = grid_for((long long)p->dim * N, kFlatPerBlock);
   for (int a = 0; a < 3; ++a) nb[BATCH_TRANSFER + a] = a < p->dim ? grid_for(p->nface_total[a], 256) : 0;
   nb[BATCH_DIVERGENCE] = g.nblk;
@@ -1526,9 +1529,6 @@ static GridDev with_rows_per_thread(GridDev g, int cr) {
 }
 constexpr int kSingleRows = 2;   // rows per thread of the sum-free single-problem divergence
 
-// Launch shape covering every cell: x over the last axis, y/z over the others.
-
-
 static bool is_device_ptr(const void *ptr) {
   if (!ptr) return true;
   cudaPointerAttributes at;
@@ -1539,7 +1539,6 @@ static bool is_device_ptr(const void *ptr) {
   return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
-// Grid-level solve: s64 (device) -> p (device, FP64), gauge applied; fills dstats fields.
 template <typename SV, typename PV>
 static void launch_residual(bool singular, bool write_r, bool norm, cudaStream_t st, const GridDev &g0,
                             const SV *s, const PV *p, float *r, DevStats *ds, double *res2, double *partials,
@@ -1578,13 +1577,6 @@ static void launch_residual(bool singular, bool write_r, bool norm, cudaStream_t
 #undef PC_RES
 }
 
-// s2 (nullable): the source as (hi, lo) pairs (projections); otherwise s64 in FP64
-// (pc_solve_poisson). FP32 solves keep the refinement iterate in p->p2 as (hi, lo) pairs, read
-// by the residual and the gradient; the last solve also writes p in FP64 to pout.
-// Gauge of the solved p: 0 none, 1 zero mean (trapezoid-weighted on the N-N axes of a vertex
-// grid: no constant part in the DCT-I expansion), 2 zero first point. Problems with a zero mode
-// take the plan's gauge: the refinement cannot correct the constant that FP32 rounding leaves
-// (L_h of a constant is zero).
 // Fluxes of axis a: every face row, or the nl listed ones that an IB node reaches (nl >= 0).
 template <bool F64>
 static void launch_transfer(const Plan *p, int a, long long nl, cudaStream_t st) {
@@ -1604,11 +1596,19 @@ static void launch_transfer(const Plan *p, int a, long long nl, cudaStream_t st)
 // transforms themselves drop the zero mode.
 static bool needs_mean(const Plan *p) { return p->singular && p->precision == PC_PREC_MIXED && p->refine_iters > 0; }
 
+// Gauge of the solved p: 0 none, 1 zero mean (trapezoid-weighted on the N-N axes of a vertex
+// grid: no constant part in the DCT-I expansion), 2 zero first point. Problems with a zero mode
+// take the plan's gauge: the refinement cannot correct the constant that FP32 rounding leaves
+// (L_h of a constant is zero).
 static int gauge_mode(const Plan *p) {
   if (!p->singular) return 0;
   return p->gauge == 1 ? 2 : 1;
 }
 
+// Grid-level solve: s64 (device) -> p (device, FP64), gauge applied; fills dstats fields.
+// s2 (nullable): the source as (hi, lo) pairs (projections); otherwise s64 in FP64
+// (pc_solve_poisson). FP32 solves keep the refinement iterate in p->p2 as (hi, lo) pairs, read
+// by the residual and the gradient; the last solve also writes p in FP64 to pout.
 static pc_status solve_grid(Plan *p, const double *s64, double *pout, bool want_final_residual,
                             cudaStream_t st, const float *s32 = nullptr, const float2 *s2 = nullptr) {
   const long long nc = p->ncells;

@@ -13,9 +13,10 @@
 //     of its forward transform, two cells per instruction, and only the rows next to other CTAs'
 //     go through global memory (in 3D all);
 //   - a sweep that the rule ended costs nothing.
-// One refined solve (two sweeps run) on a GB300, before (one launch per pass and residual) and
-// now: 128^2 102 -> 59 us, 512^2 156 -> 76, 1024 x 512 about 140 -> 80, 1024^2 258 -> 135, 96^3
-// 261 -> 199. A phase of the 1024 x 512 grid takes about 7 us: five half-stages per transform at
+// One call of the solve with walls on every side (two sweeps run; the sum of the source and the gauge with
+// it) on a GB300, before (one launch per pass and residual) and now: 128^2 104 -> 55 us, 512^2 156 -> 75,
+// 1024 x 512 217 -> 96, 1024^2 274 -> 159, 96^3 268 -> 193; with an outlet 128^2 43, 512^2 59, 1024 x 512 78.
+// A phase of the 1024 x 512 grid takes about 7 us: five half-stages per transform at
 // 0.35 us each (latency and issue alike: 38% of the issue slots), 1 us to load, 1 to store, the
 // barrier.
 #include <atomic>
@@ -217,7 +218,7 @@ __global__ void __launch_bounds__(kResidentThreads, 1) resident_kernel(const __g
       for (int tile = t0; tile < t1; tile += step) {
         if (tile != t0) __syncthreads();   // the previous tile's outputs have left the buffers
         const int d0 = (tile - t0) * A.L;
-        loop::pass_tile<float, true, IEEE>(
+        loop::pass_tile<float, IEEE>(
             A, tile, buf, tb, w16tab,
             [&](int l, int base, int qd, int stride) -> Quad<float> {
               if (!first) return loop::load_src4<float>(src, SRC_WORK, base + 4 * qd * stride, stride);

@@ -69,7 +69,7 @@ __global__ void __launch_bounds__(kResidentThreads, 1) resident64_kernel(const _
     for (int tile = t0; tile < t1; tile += step) {
       if (tile != t0) __syncthreads();
       const int d0 = (tile - t0) * A.L;
-      loop::pass_tile<double, true, false>(
+      loop::pass_tile<double, false>(
           A, tile, buf, tb, w16tab,
           [&](int, int base, int qd, int stride) { return loop::load_src4<double>(src, SRC_WORK, base + 4 * qd * stride, stride); },
           [&](int l, int base, int qd, int stride, const Quad<double> &x) {
