@@ -3,6 +3,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <vector>
 
 #include "pc_internal.cuh"
@@ -104,6 +105,36 @@ void plan_drop_graphs(Plan *p) {
   }
 }
 
+// The plans' host words: 1024 in one pinned page that the process keeps (pinning one per plan took 300 us,
+// as long as a small grid plan), further ones pinned for their plan.
+constexpr int kWords = 1024;
+static std::mutex g_words_mutex;
+static unsigned *g_words = nullptr;
+static std::vector<int> g_free_words;
+
+static pc_status take_word(unsigned **out) {
+  std::lock_guard<std::mutex> lock(g_words_mutex);
+  if (!g_words) {
+    PC_CUDA_TRY(cudaHostAlloc((void **)&g_words, kWords * sizeof(unsigned), cudaHostAllocPortable));
+    for (int i = kWords - 1; i >= 0; --i) g_free_words.push_back(i);
+  }
+  if (g_free_words.empty()) {
+    PC_CUDA_TRY(cudaHostAlloc((void **)out, sizeof(unsigned), cudaHostAllocPortable));
+  } else {
+    *out = g_words + g_free_words.back();
+    g_free_words.pop_back();
+  }
+  **out = 0u;
+  return PC_OK;
+}
+
+static void give_word(unsigned *w) {
+  if (!w) return;
+  std::lock_guard<std::mutex> lock(g_words_mutex);
+  if (w >= g_words && w < g_words + kWords) g_free_words.push_back((int)(w - g_words));
+  else cudaFreeHost(w);
+}
+
 pc_status wait_status(Plan *p) {
   if (!p->gave_up || !__atomic_exchange_n(p->gave_up, 0u, __ATOMIC_ACQ_REL)) return PC_OK;
   return fail(PC_ERR_TIMEOUT, "a wait inside a solve of this plan gave up: its pressure holds NaN");
@@ -129,7 +160,7 @@ static void destroy_plan(Plan *p) {
     if (p->copy_ev[e]) cudaEventDestroy(p->copy_ev[e]);
   if (p->ib_body_stream) cudaStreamDestroy(p->ib_body_stream);
   for (int i = 0; i < p->nallocs; ++i) cudaFree(p->allocs[i]);
-  if (p->gave_up) cudaFreeHost(p->gave_up);
+  give_word(p->gave_up);   // the frees above waited for the kernels that may set it
   if (cur >= 0) cudaSetDevice(cur);
   delete p;
 }
@@ -219,9 +250,7 @@ static pc_status alloc_workspace(Plan *p, cudaStream_t st) {
   if (cudaMemsetAsync(p->counters, 0, 16 * sizeof(unsigned int), st) != cudaSuccess ||
       cudaMemsetAsync(p->dstats, 0, sizeof(DevStats), st) != cudaSuccess)
     return fail(PC_ERR_CUDA, "counter reset failed");
-  if (cudaHostAlloc((void **)&p->gave_up, sizeof(unsigned), cudaHostAllocPortable) != cudaSuccess)
-    return fail(PC_ERR_CUDA, "host word allocation failed");
-  *p->gave_up = 0u;
+  PC_TRY(take_word(&p->gave_up));
   if (cudaStreamCreateWithFlags(&p->cap_stream, cudaStreamNonBlocking) != cudaSuccess)
     return fail(PC_ERR_CUDA, "stream creation failed");
   for (int e = 0; e < kProfEvents; ++e)

@@ -83,6 +83,27 @@ def test_other_calls_report_it(pc):
     other.close()
 
 
+@pytest.mark.gpu
+def test_more_plans_than_pooled_words(pc):
+    """Each plan reports its own waits, also those beyond the 1024 whose words share a page."""
+    small = [pc.GridPlan(2, (8, 8), (1 / 8, 1 / 8), "WW", "WW") for _ in range(1023)]
+    plans = [pc.GridPlan(2, N, H, "IW", "DW") for _ in range(3)]
+    s = _source()
+    want = plans[0].solve_poisson(s)[0].clone()
+    for plan in (plans[0], plans[2]):
+        plan.set_wait_limit(1)
+        plan.solve_poisson(s)
+    torch.cuda.synchronize()
+    _timeout(pc, lambda: plans[0].solve_poisson(s))
+    assert torch.equal(plans[1].solve_poisson(s)[0], want)
+    _timeout(pc, lambda: plans[2].solve_poisson(s))
+    for plan in small + plans:
+        plan.close()
+    plan = pc.GridPlan(2, N, H, "IW", "DW")
+    assert torch.equal(plan.solve_poisson(s)[0], want)
+    plan.close()
+
+
 # one cluster and cooperative grids in 2D and 3D, both gauges
 @pytest.mark.gpu
 @pytest.mark.parametrize("n,lo,hi,gauge", [((64, 64), "WP", "WP", 0), ((48, 64), "ID", "WD", 0), ((64, 60), "WW", "WW", 1),
