@@ -246,12 +246,12 @@ def measured_peaks():
 
 
 def transform_kernel_hash():
-    """Hash of the transform kernels' device code (fft.cuh, axis_pass.cuh, lean_pass.cuh) with
-    whole-line comments and blank lines left out, so host-only edits and comment edits keep a
-    capture valid."""
+    """Hash of the code of the one-launch solve that the timed projection runs (resident.cu and what it
+    is made of) with whole-line comments and blank lines left out, so that edits elsewhere and comment
+    edits keep a capture valid."""
     csrc = os.path.join(ROOT, "paper_2304_14690_gb300", "csrc")
     h = hashlib.sha1()
-    for f in ("fft.cuh", "axis_pass.cuh", "lean_pass.cuh"):
+    for f in ("fft.cuh", "pairs.cuh", "dfloat.cuh", "loop_pass.cuh", "resident.cu", "resident.cuh"):
         for line in open(os.path.join(csrc, f), encoding="utf-8"):
             t = line.strip()
             if t and not t.startswith("//"):
