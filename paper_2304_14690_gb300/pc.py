@@ -348,7 +348,7 @@ class Plan:
 
     def set_slots(self, axis, slots, precision=None):
         """Slots per thread of the transform passes along axis (2, 4, 8 or 16; for FP32 passes
-        also 0, the default, and 1: see pc_plan_set_transform_slots)."""
+        also 0 and 1; the defaults are 0 and, in FP64, 2: see pc_plan_set_transform_slots)."""
         _check(load().pc_plan_set_transform_slots(self.handle, axis, self._prec_code(precision), slots))
 
     def slots(self, precision=None):
@@ -361,7 +361,7 @@ class Plan:
         return out
 
     def set_ctas(self, axis, ctas_per_sm, precision=None):
-        """CTAs per SM the single-problem passes along axis aim for (1, 2, 4 or 8)."""
+        """CTAs per SM the general single-problem passes along axis aim for (1, 2, 4 or 8)."""
         _check(load().pc_plan_set_transform_ctas(self.handle, axis, self._prec_code(precision), ctas_per_sm))
 
     def ctas(self, precision=None):
