@@ -501,8 +501,8 @@ constexpr int kSpreadSlots = 512;
 
 // Tiles, tables and own rows of a cooperative solve's passes: lines per tile as few as give every SM
 // at most one tile, more while the tile has no more than `spread` slots, and fewer again where the
-// buffers would not leave room for the own rows (own_bytes per cell). Behind the tiles: per axis the wrappers' factors its family reads, the stage
-// twiddles and, on the dividing pass, the eigenvalues.
+// buffers would not leave room for the own rows (own_bytes per cell). Behind the tiles: per axis the
+// wrappers' factors its family reads, the stage twiddles and, on the dividing pass, the eigenvalues.
 template <typename Real>
 static bool resident_layout(const Plan *p, const std::vector<PassSpec> &specs, PassArgs<Real> *pass, int sms, int spread,
                             int cap0, int own_bytes, int &grid, int &row_tiles, int &tables_at, int &own_at, size_t &smem) {
@@ -528,9 +528,12 @@ static bool resident_layout(const Plan *p, const std::vector<PassSpec> &specs, P
     for (int k = 0; k < np; ++k) {
       const int M = p->ax[specs[k].axis].M;
       const long long lines = p->ncells / p->ax[specs[k].axis].n;
+      long long run = 1;   // lines side by side: a column tile's do not go beyond
+      for (int b = specs[k].axis + 1; b < p->dim; ++b) run *= p->n[b];
+      if (specs[k].axis == last) run = lines;
       int L = 1;
       while ((lines + L - 1) / L > sms && 2 * L * M <= cap) L *= 2;
-      while (2 * L * M <= spread) L *= 2;
+      while (L < run && 2 * L * M <= spread) L *= 2;
       const long long tiles = fill_loop<Real>(p, specs[k], pass[k], L);
       most = tiles > most ? tiles : most;
       const size_t b = loop::tile_smem<Real>(M, L);

@@ -25,7 +25,7 @@ static bool valid_ctas(int c) { return c == 1 || c == 2 || c == 4 || c == 8; }
 // Sweeps of the timed solve: a refined plan's first two, which is what the stopping rule mostly leaves.
 // Without them the 1024 x 512 channel's one-launch solve (31 us for one solve) could lose to launches of
 // variant 1 (25), which take 185 us per projection against 129. Grids beyond that solve time one solve
-// (256x128x128 box: tuned in 0.09 s, with the sweeps in 0.15).
+// (256x128x128 box: tuned in 0.073 s, with the sweeps in 0.103).
 static int tuned_sweeps(const Plan *p) {
   if (p->precision != PC_PREC_MIXED || p->ncells > kResidentCells) return 0;
   return p->refine_iters < 2 ? p->refine_iters : 2;

@@ -108,7 +108,11 @@ def test_more_plans_than_pooled_words(pc):
 @pytest.mark.gpu
 @pytest.mark.parametrize("n,lo,hi,gauge", [((64, 64), "WP", "WP", 0), ((48, 64), "ID", "WD", 0), ((64, 60), "WW", "WW", 1),
                                            ((12, 16, 20), "WWW", "WWW", 0), (N, "WW", "WW", 0), ((400, 200), "PP", "PP", 1),
-                                           ((48, 40, 60), "WPW", "WPW", 0), ((64, 48, 32), "DPW", "WPD", 0)])
+                                           ((48, 40, 60), "WPW", "WPW", 0), ((64, 48, 32), "DPW", "WPD", 0),
+                                           # many short lines, tiles wider than the lines side by side
+                                           ((2048, 16), "IW", "DW", 0), ((16, 2048), "WD", "WW", 0), ((1200, 20), "PW", "PW", 0),
+                                           ((400, 12, 12), "WWP", "WWP", 0), ((12, 200, 12), "DIP", "WDP", 0),
+                                           ((32, 32, 32), "WWW", "WWW", 0)])
 def test_without_waits(pc, n, lo, hi, gauge):
     """Limit 0: one launch per pass. Mixed solves keep their bits, and FP64 ones without a zero mode;
     with one, the gauge constant of the launches is summed as FP32 pairs (each thread's sum cut to
