@@ -34,7 +34,6 @@ struct PassLaunch {
   int emax = 1;          // largest slots per thread among the items' passes (kernel instance)
   size_t smem = 0;       // the pass body's shared memory (the largest item's)
   int lean = 0;          // 0: general passes; 1-6 the lean kernel id (lean_pass.cuh); 7 looped passes
-  bool ieee = false;     // looped passes: some divide with IEEE rounding
   int pass = 0;          // the pass of the solve: launches of one pass run side by side
 };
 
@@ -96,6 +95,7 @@ struct Exec {
   PassArgs<float> *dargs = nullptr;     // transform passes of every problem and solve
   int4 *ditems = nullptr;               // work list: (args index, first tile, tiles, 0)
   std::vector<std::vector<PassLaunch>> passes;   // [solve][pass]
+  bool ieee = false;                    // some looped pass divides to nearest: its instance for all
   cudaStream_t cap = nullptr;
   Fork own;                             // streams of the side-by-side pass launches (cached executors)
   Fork *fork = nullptr;                 // the streams used: own, or the batch executor's
@@ -224,7 +224,7 @@ pc_status build_passes(Exec *e) {
         pl[c].smem = std::max(pl[c].smem, smem);
         pl[c].emax = std::max(pl[c].emax, A.emax);
         pl[c].lean = c;
-        pl[c].ieee = pl[c].ieee || (A.do_div && A.ieee_div);
+        if (A.loop && A.do_div && A.ieee_div) e->ieee = true;
         pl[c].pass = (int)k;
       }
       for (int c = 0; c < 8; ++c) {
@@ -304,7 +304,7 @@ pc_status record_exec(Exec *e, cudaStream_t st, Plan *prof = nullptr) {
         PassArgs<float> none;
         memset(&none, 0, sizeof(none));
         if (pl.lean == 7) {
-          PC_TRY(launch_loop(none, e->dargs, e->ditems + pl.items_off, (unsigned)pl.nitems, pl.smem, pl.ieee, ls));
+          PC_TRY(launch_loop(none, e->dargs, e->ditems + pl.items_off, (unsigned)pl.nitems, pl.smem, e->ieee, ls));
         } else if (pl.lean) {
           PC_TRY(launch_lean(pl.lean, none, e->dargs, e->ditems + pl.items_off, (unsigned)pl.nitems, kBatchThreads, pl.smem, ls));
         } else {

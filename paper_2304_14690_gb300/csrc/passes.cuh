@@ -47,10 +47,11 @@ struct PassArgs {
   int chunk;            // single-problem launches: consecutive tiles per CTA (>= 1)
   int ntiles;           // tiles of the pass
   int lean;             // 0: general pass (axis_pass.cuh); else the lean kernel id (lean_pass.cuh)
-  // looped passes (loop_pass.cuh): transform family, slots between the lines of a tile, IEEE division,
+  // looped passes (loop_pass.cuh): transform family, slots between the lines of a tile, division to nearest,
   // 2^32 / (M/2) rounded up, and the stage twiddles (StageInfo::stride_m is a stage's offset in them)
   int loop, fam, ls, ieee_div;
   unsigned half_magic;
+  Real div_scale;       // power of two on the divisors (the quotients' is in out_scale)
   const T *stw;
   // the resident kernel's copies in shared memory: slots [tw_first, tw_last) of the table at tw_at,
   // stage twiddles at st_at (both in slots), eigenvalues at lam_at (in values)
@@ -121,8 +122,8 @@ pc_status prepare_lean_r1f1(int lim);
 pc_status launch_lean_r1f2(const PassArgs<float> &A, const PassArgs<float> *dargs, const int4 *ditems,
                             unsigned grid, int threads, size_t smem, cudaStream_t st);
 pc_status prepare_lean_r1f2(int lim);
-// Looped passes (loop_pass.cuh), single-problem (dargs == ditems == nullptr) and batched (FP32). ieee: some
-// of the passes divide with IEEE rounding.
+// Looped passes (loop_pass.cuh), single-problem (dargs == ditems == nullptr) and batched (FP32). ieee: the
+// instance for solves that divide to nearest (PassArgs::ieee_div).
 pc_status launch_loop(const PassArgs<float> &A, const PassArgs<float> *dargs, const int4 *ditems, unsigned grid,
                       size_t smem, bool ieee, cudaStream_t st);
 pc_status launch_loop(const PassArgs<double> &A, unsigned grid, size_t smem, cudaStream_t st);

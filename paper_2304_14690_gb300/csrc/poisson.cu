@@ -237,6 +237,13 @@ static long long fill_loop(const Plan *p, const PassSpec &ps, PassArgs<Real> &A,
   A.loop = 1;
   A.fam = pass_family(ax.kind);
   A.ieee_div = !lean::length_ok(ax.M);   // lengths with a compile-time pass keep its division, and its bits
+  A.div_scale = 1;
+  if (sizeof(Real) == 4 && ps.div && A.ieee_div) {
+    double top = 0.0;   // of the eigenvalue sums, FD or spectral
+    for (int a = 0; a < p->dim; ++a) top += 9.87 / (p->h[a] * p->h[a]);
+    A.div_scale = (Real)(top > 0x1p100 ? 0x1p-64 : (top < 0x1p-60 ? 0x1p64 : 1.0));
+    A.out_scale *= A.div_scale;
+  }
   A.nst = ax.loop_nst;
   for (int s = 0; s < ax.loop_nst; ++s) A.st[s] = ax.loop_st[s];
   A.stw = A.tw + tw_total(ax.M);
@@ -402,7 +409,8 @@ static pc_status launch_pass(Plan *p, const PassSpec &ps, cudaStream_t st) {
   PC_TRY(build_pass<Real>(p, ps, A, tiles, threads, smem, 0));
   tiles = (tiles + A.chunk - 1) / A.chunk;   // CTAs
   if (A.loop) {
-    if constexpr (sizeof(Real) == 4) PC_TRY(launch_loop(A, nullptr, nullptr, (unsigned)tiles, smem, A.do_div && A.ieee_div, st));
+    // one instance for all passes of a solve: its code stays in the instruction caches
+    if constexpr (sizeof(Real) == 4) PC_TRY(launch_loop(A, nullptr, nullptr, (unsigned)tiles, smem, !lean::length_ok(p->ax[0].M), st));
     else PC_TRY(launch_loop(A, (unsigned)tiles, smem, st));
     count_launch(p);
     return PC_OK;

@@ -160,7 +160,7 @@ __device__ __forceinline__ void cta_max(float v, float *dst) {
   }
 }
 
-// IEEE: the pass of axis 0 divides with IEEE rounding (PassArgs::ieee_div).
+// IEEE: the pass of axis 0 divides to nearest (PassArgs::ieee_div).
 template <int DIM, typename SV, bool CLUSTER, bool IEEE>
 __global__ void __launch_bounds__(kResidentThreads, 1) resident_kernel(const __grid_constant__ ResidentArgs R) {
   constexpr int NP = 2 * DIM - 1;
