@@ -2021,8 +2021,9 @@ static pc_status vertex_solve(Plan *p, const double *s, double *p_out, pc_stats 
   PC_CUDA_TRY(cudaGetLastError());
   if (hp) PC_CUDA_TRY(cudaMemcpyAsync(p_out, dp, nc * sizeof(double), cudaMemcpyDeviceToHost, st));
   if (stats) PC_TRY(fill_stats(p, stats, st));
-  if (hp) PC_CUDA_TRY(cudaStreamSynchronize(st));
-  return PC_OK;
+  if (!hp) return PC_OK;
+  PC_CUDA_TRY(cudaStreamSynchronize(st));
+  return wait_status(p);
 }
 
 static pc_status solve_impl(Plan *p, const double *s, double *p_out, pc_stats *stats, cudaStream_t st,

@@ -84,6 +84,20 @@ def test_other_calls_report_it(pc):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("precision", ["mixed", "fp64"])
+def test_periodic_vertex_grid(pc, precision):
+    """A vertex grid of periodic axes has the cell grid's transforms, and its waits."""
+    plan = pc.GridPlan(2, N, H, "PP", "PP", grid_type="vertices", precision=precision)
+    s = _source()
+    want = plan.solve_poisson(s)[0].clone()
+    plan.set_wait_limit(1)
+    _timeout(pc, lambda: plan.solve_poisson(s.cpu()))
+    plan.set_wait_limit(1 << 22)
+    assert torch.equal(plan.solve_poisson(s)[0], want)
+    plan.close()
+
+
+@pytest.mark.gpu
 def test_more_plans_than_pooled_words(pc):
     """Each plan reports its own waits, also those beyond the 1024 whose words share a page."""
     small = [pc.GridPlan(2, (8, 8), (1 / 8, 1 / 8), "WW", "WW") for _ in range(1023)]
